@@ -25,10 +25,19 @@
 
 namespace lbm {
 
-template <class R>
-struct BatchMember {
+// What the reduced step needs of a member, for the storage forms that have one.
+template <class S, bool = has_unit_step_2d<S>::value>
+struct BatchUnit {
+    UnitCoeffs<typename S::R> u;
+    int unit;                 // the member takes the reduced collision (unit_rates_2d)
+};
+template <class S>
+struct BatchUnit<S, false> {};
+
+template <class S>
+struct BatchMember : BatchUnit<S> {
     Geometry geo;
-    Coeffs2D<R> c;
+    Coeffs2D<typename S::R> c;
     unsigned long long off;   // element offset of the member's planes in the f and g buffers
     int tile0;                // first global tile index of the member
     int tiles_x;              // tiles along x
@@ -45,10 +54,10 @@ template <class S>
 __global__ void __launch_bounds__(256, BatchBounds<S>::kMinBlocks)
     batch_step_d2q9_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                            typename S::T* __restrict__ fout, typename S::T* __restrict__ gout,
-                           const BatchMember<typename S::R>* __restrict__ members, int n_members,
+                           const BatchMember<S>* __restrict__ members, int n_members,
                            int n_tiles, int tile_x, int tile_y, unsigned* status)
 {
-    using M = BatchMember<typename S::R>;
+    using M = BatchMember<S>;
     __shared__ __align__(16) unsigned char mbuf[sizeof(M)];
     const M& m = *reinterpret_cast<const M*>(mbuf);
     // block b owns the contiguous tile range [t0, t1): equal shares, the first `rem` blocks one more
@@ -76,9 +85,16 @@ __global__ void __launch_bounds__(256, BatchBounds<S>::kMinBlocks)
         const int local = t - m.tile0;
         const int x = (local % m.tiles_x) * tile_x + (int)threadIdx.x % tile_x;
         const int y = (local / m.tiles_x) * tile_y + (int)threadIdx.x / tile_x;
-        if (x < m.geo.nx && y < m.geo.ny)
-            node_step_d2q9<S, unsigned>(fin + m.off, gin + m.off, fout + m.off, gout + m.off, m.geo, m.c,
-                                        status + k, x, y);
+        if (x >= m.geo.nx || y >= m.geo.ny) continue;
+        if constexpr (has_unit_step_2d<S>::value) {
+            if (m.unit) {
+                node_step_d2q9<S, unsigned, true>(fin + m.off, gin + m.off, fout + m.off, gout + m.off,
+                                                  m.geo, m.u, status + k, x, y);
+                continue;
+            }
+        }
+        node_step_d2q9<S, unsigned>(fin + m.off, gin + m.off, fout + m.off, gout + m.off, m.geo, m.c,
+                                    status + k, x, y);
     }
 }
 
@@ -102,7 +118,7 @@ static cudaError_t launch_batch(const void* fin, const void* gin, void* fout, vo
     using T = typename S::T;
     batch_step_d2q9_kernel<S><<<grid, tile_x * tile_y, 0, st>>>(
         (const T*)fin, (const T*)gin, (T*)fout, (T*)gout,
-        (const BatchMember<typename S::R>*)members, n_members, n_tiles, tile_x, tile_y, status);
+        (const BatchMember<S>*)members, n_members, n_tiles, tile_x, tile_y, status);
     return cudaGetLastError();
 }
 
@@ -177,10 +193,11 @@ void brelease(lbm_batch_s* b)
     delete b;
 }
 
-template <class R>
-std::vector<lbm::BatchMember<R>> member_table(const lbm_batch_s* b)
+template <class S>
+std::vector<lbm::BatchMember<S>> member_table(const lbm_batch_s* b)
 {
-    std::vector<lbm::BatchMember<R>> t(b->count);
+    using R = typename S::R;
+    std::vector<lbm::BatchMember<S>> t(b->count);
     int tile = 0;
     for (int k = 0; k < b->count; ++k) {
         const lbm::BoxPlan& P = b->plans[k];
@@ -189,38 +206,39 @@ std::vector<lbm::BatchMember<R>> member_table(const lbm_batch_s* b)
         t[k].off = b->off[k];
         t[k].tile0 = tile;
         t[k].tiles_x = (P.nx + b->tile_x - 1) / b->tile_x;
+        if constexpr (lbm::has_unit_step_2d<S>::value) {
+            t[k].u = lbm::make_unit_coeffs<R, 2>(P.hc);
+            t[k].unit = lbm::unit_rates_2d(P.hc) ? 1 : 0;
+        }
         tile += t[k].tiles_x * ((P.ny + b->tile_y - 1) / b->tile_y);
     }
     return t;
 }
 
-// Upload the member table for the current tile shape.
-int upload_table(lbm_batch_s* b)
+template <class S>
+int upload_table_as(lbm_batch_s* b)
 {
-    size_t bytes = 0;
-    const void* src = nullptr;
-    std::vector<lbm::BatchMember<double>> td;
-    std::vector<lbm::BatchMember<float>> tf;
-    if (b->prec == lbm::kF64) {
-        td = member_table<double>(b);
-        bytes = td.size() * sizeof(td[0]);
-        src = td.data();
-        b->n_tiles = td.back().tile0 + td.back().tiles_x * ((b->plans.back().ny + b->tile_y - 1) / b->tile_y);
-    } else {
-        tf = member_table<float>(b);
-        bytes = tf.size() * sizeof(tf[0]);
-        src = tf.data();
-        b->n_tiles = tf.back().tile0 + tf.back().tiles_x * ((b->plans.back().ny + b->tile_y - 1) / b->tile_y);
-    }
+    const auto t = member_table<S>(b);
+    const size_t bytes = t.size() * sizeof(t[0]);
+    b->n_tiles = t.back().tile0 + t.back().tiles_x * ((b->plans.back().ny + b->tile_y - 1) / b->tile_y);
     if (!b->members) {
-        const size_t cap = (size_t)b->count * std::max(sizeof(lbm::BatchMember<double>), sizeof(lbm::BatchMember<float>));
-        b->members = b->alloc(cap, b->actx);
+        b->members = b->alloc(bytes, b->actx);
         if (!b->members) return bfail(b, LBM_ENOMEM, "no device memory for the member table");
     }
-    B_CK(b, cudaMemcpyAsync(b->members, src, bytes, cudaMemcpyHostToDevice, b->stream));
+    B_CK(b, cudaMemcpyAsync(b->members, t.data(), bytes, cudaMemcpyHostToDevice, b->stream));
     B_CK(b, cudaStreamSynchronize(b->stream));
     ++b->gen;
     return LBM_OK;
+}
+
+// Upload the member table for the current tile shape.
+int upload_table(lbm_batch_s* b)
+{
+    switch (b->prec) {
+    case lbm::kF64: return upload_table_as<lbm::StoreF64>(b);
+    case lbm::kF32: return upload_table_as<lbm::StoreF32>(b);
+    default: return upload_table_as<lbm::StoreF16S>(b);
+    }
 }
 
 int max_resident(int prec, int threads);

@@ -7,6 +7,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "lattices.cuh"
 #include "lbm_common.cuh"
 #include "../../include/lbm.h"
 #include <string>
@@ -144,6 +145,22 @@ inline Coeffs<R, QF, QG> make_coeffs(const HostCoeffs& h)
     return c;
 }
 
+template <class R, int DIM>
+inline UnitCoeffs<R> make_unit_coeffs(const HostCoeffs& h)
+{
+    UnitCoeffs<R> c{};
+    for (int a = 4; a < 10; ++a) c.kf[a - 4] = a < (DIM == 2 ? 9 : 27) ? R(1.0 - h.om_f[a]) : R(0);
+    for (int b = 1; b < 4; ++b) c.kg[b - 1] = R(1.0 - h.om_g[b]);
+    c.gbeta = R(h.gbeta);
+    c.T_ref = R(h.T_ref);
+    c.T_ref6 = R(h.T_ref / 6.0);
+    c.T_ref23 = R(h.T_ref * (2.0 / 3.0));
+    const double w[3] = {DIM == 2 ? w9(0) : w15(0), DIM == 2 ? w9(1) : w15(1), DIM == 2 ? w9(8) : w15(14)};
+    for (int k = 0; k < 3; ++k) c.wT[k] = R(w[k]) * R(h.T_ref);
+    c.fp16_sr = h.fp16_sr;
+    return c;
+}
+
 // Default thread blocks, x-major so that a warp reads and writes 32 consecutive nodes; a
 // caller-chosen shape (block.x > 0) replaces it.  2D: 256 threads.  3D: 64 x 1, which at 96
 // registers per thread lets 10 blocks (20 warps) share an SM against 16 warps for 256-thread
@@ -185,6 +202,16 @@ inline bool unit_flow_rates(const HostCoeffs& h)
 {
     for (int a = 0; a < 27; ++a)
         if (!(a >= 4 && a <= 6) && a != 8 && a != 9 && h.om_f[a] != 1.0) return false;
+    return true;
+}
+
+// The 2D box takes the reduced collision (collide_store_d2q9_unit): option A, every rate 1 except the
+// shear (flow slots 4, 5) and diffusivity (energy slots 1, 2) ones, gravity along y.
+inline bool unit_rates_2d(const HostCoeffs& h)
+{
+    if (h.gopt != 0 || h.gaxis != 1) return false;
+    for (int a = 0; a < 9; ++a)
+        if ((a != 4 && a != 5 && h.om_f[a] != 1.0) || (a != 1 && a != 2 && h.om_g[a] != 1.0)) return false;
     return true;
 }
 

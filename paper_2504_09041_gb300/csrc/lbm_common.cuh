@@ -24,9 +24,17 @@ enum FaceKind { kPeriodic = 0, kAdiabatic = 1, kFixedT = 2 };
 //  - F16S stores the deviations scaled by 2^10, so that deviations down to 6e-8 stay in FP16's
 //    normal range (full 11-bit significand) while |deviation| < 64 still fits; the scale is a
 //    power of two and adds no rounding.
+//
+// The reduced steps (default rates and gravity axis) take the stored number itself (load_raw) and
+// work in its units: every relation of the step is homogeneous of degree one in the populations, so
+// multiplying them all by kUnits only multiplies the rest state's constants.  kFull: the stored
+// number is the population, not its deviation; the rest state is then taken off in the raw sums.
 struct StoreF64 {
     using T = double;
     using R = double;
+    static constexpr bool kFull = true;
+    static constexpr double kUnits = 1.0;
+    __device__ static R load_raw(const T* p, size_t i) { return __ldg(p + i); }
     __device__ static R load_dev(const T* p, size_t i, R shift) { return __ldg(p + i) - shift; }
     __device__ static void store_dev(T* p, size_t i, R dev, R shift) { p[i] = shift + dev; }
 };
@@ -49,6 +57,9 @@ __device__ __forceinline__ __half ldg_pf256(const __half* p)
 struct StoreF32 {
     using T = float;
     using R = float;
+    static constexpr bool kFull = false;
+    static constexpr double kUnits = 1.0;
+    __device__ static R load_raw(const T* p, size_t i) { return ldg_pf256(p + i); }
     __device__ static R load_dev(const T* p, size_t i, R) { return ldg_pf256(p + i); }
     __device__ static void store_dev(T* p, size_t i, R dev, R) { p[i] = dev; }
 };
@@ -58,6 +69,9 @@ struct StoreF16S {
     static constexpr int kScaleLog2 = 10;
     static constexpr float kScale = 1024.0f;   // 2^kScaleLog2
     static constexpr float kInvScale = 1.0f / 1024.0f;
+    static constexpr bool kFull = false;
+    static constexpr double kUnits = 1024.0;
+    __device__ static R load_raw(const T* p, size_t i) { return __half2float(ldg_pf256(p + i)); }
     __device__ static R load_dev(const T* p, size_t i, R)
     {
         return __half2float(ldg_pf256(p + i)) * kInvScale;
@@ -132,6 +146,18 @@ struct Coeffs {
     int gaxis;    // 0, 1, 2
     int gopt;     // energy attractors of orders 3-4: 0 = option A, 1 = option B (renormalized)
     int fp16_sr;  // F16S storage: 1 = stochastic rounding of the stored deviations, 0 = nearest
+};
+
+// What the reduced steps (default rates and gravity axis) take instead, formed once on the host: their
+// FP64 pipe is their bound, so no constant is formed per thread.
+template <class R>
+struct UnitCoeffs {
+    R kf[6];             // 1 - omega of flow slots 4 .. 9
+    R kg[3];             // 1 - omega of energy slots 1 .. 3
+    R gbeta, T_ref;
+    R T_ref6, T_ref23;   // T_ref / 6 and 2 T_ref / 3: the rest state's share of an outer and a middle line
+    R wT[3];             // rest weights of the energy (centre, axis, corner links) times T_ref
+    int fp16_sr;         // as in Coeffs
 };
 
 // Per-thread wall bookkeeping for the pull.  For an axis, "m" is a link whose source lies at
@@ -253,6 +279,49 @@ __device__ __forceinline__ int link_source(const Geometry& g, const NodeWalls<R>
     return s;
 }
 
+// Stored numbers at one link, for a population (load_dev) or in storage units (load_raw).
+template <class S, bool kRaw, class Idx>
+__device__ __forceinline__ typename S::R load_link(const typename S::T* p, Idx off, typename S::R shift)
+{
+    if constexpr (kRaw) return S::load_raw(p, off);
+    else return S::load_dev(p, off, shift);
+}
+// Anti-bounce-back of the energy population gv against a wall at temperature tw (link weight w), in
+// the units of load_link.
+template <class S, bool kRaw>
+__device__ __forceinline__ typename S::R anti_bounce(typename S::R gv, double w, typename S::R tw,
+                                                     typename S::R T_ref)
+{
+    using R = typename S::R;
+    if constexpr (kRaw && S::kFull) return R(2.0 * w) * tw - gv;
+    else if constexpr (kRaw) return R(2.0 * S::kUnits * w) * (tw - T_ref) - gv;
+    else return R(2.0 * w) * (tw - T_ref) - gv;
+}
+
+// One line of an inverse sweep whose moments of order 1 and 2 come in halved (h1, h2) and whose
+// order-0 moment is split into a constant and the rest k0: (k0 + const, 2 h1, 2 h2 + const / 3) at
+// velocity u -> the deviations of the three links from the constant's rest weights.  k0f is the full
+// order-0 moment and uh = u / 2.  Six operations; the halvings of uncentral_line are carried by the
+// inputs instead (exact: powers of two).
+template <class R>
+__device__ __forceinline__ void unline(R k0, R k0f, R h1, R h2, R u, R uh, R& a, R& b, R& c)
+{
+    const R r1 = h1 + uh * k0f;           // half the raw first moment
+    const R r2 = h2 + u * (h1 + r1);      // half the raw second moment (deviation)
+    a = r2 - r1;
+    b = k0 - R(2) * r2;
+    c = r2 + r1;
+}
+// The same with a zero order-0 moment; u2 = 2 u.
+template <class R>
+__device__ __forceinline__ void unline0(R h1, R h2, R u2, R& a, R& b, R& c)
+{
+    const R r2 = h2 + u2 * h1;
+    a = r2 - h1;
+    b = R(-2) * r2;
+    c = r2 + h1;
+}
+
 // Compile-time loop: calls f(std::integral_constant<int, 0>), ..., f(<N-1>).
 template <class F, int... Is>
 __device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, Is...>)
@@ -294,12 +363,42 @@ __device__ __forceinline__ void store_node_f16s_sr(__half* __restrict__ fout, __
     });
 }
 
+// 1 / x to about an ulp: the hardware's approximation y and one step of a power series in its residual
+// e = 1 - x y: 1 / x = y (1 + e + e^2 + ...), to order e^2 for double (y has about 20 bits) and to order
+// e for float.  Three FP64 operations instead of the eight or so of an IEEE division, whose last
+// half ulp the velocity does not need.
+__device__ __forceinline__ double recip(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float recip(float x)
+{
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return fmaf(y, fmaf(-x, y, 1.0f), y);
+}
+
 // Divergence flag: bit 0 set when a node sees a non-finite or non-positive density or a
 // non-finite temperature.
 template <class R>
 __device__ __forceinline__ void check_node(unsigned* status, R rho, R T)
 {
     if (!(rho > R(0)) || !(fabs(T) < R(1e30)) || !(rho < R(1e30))) atomicOr(status, 1u);
+}
+
+// The same test of FP64 values on their bits, off the FP64 pipe: 0x46293e59 is the high word of 1e30.
+__device__ __forceinline__ void check_node_bits(unsigned* status, double rho, double T)
+{
+    const int hr = __double2hiint(rho), ht = __double2hiint(T) & 0x7fffffff;
+    const bool positive = hr > 0 || (hr == 0 && __double2loint(rho) != 0);
+    if (!positive || hr >= 0x46293e59 || ht >= 0x46293e59) atomicOr(status, 1u);
+}
+__device__ __forceinline__ void check_node_bits(unsigned* status, float rho, float T)
+{
+    check_node(status, rho, T);
 }
 
 }  // namespace lbm

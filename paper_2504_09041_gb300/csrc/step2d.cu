@@ -4,22 +4,34 @@
 
 namespace lbm {
 
-template <class S>
-static cudaError_t run(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
-                       const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
+template <class S, bool kUnit>
+static cudaError_t run_as(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
+                          const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
 {
     using T = typename S::T;
     using R = typename S::R;
     const dim3 b = block_shape(geo.nx, block);
     const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
-    const auto c = make_coeffs<R, 9, 9>(hc);
+    StepCoeffs2D<S, kUnit> c;
+    if constexpr (kUnit) c = make_unit_coeffs<R, 2>(hc);
+    else c = make_coeffs<R, 9, 9>(hc);
     if (step_index32(geo, 9, hc))
-        step_d2q9_kernel<S, unsigned><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
-                                                          (T*)gout, geo, c, status);
+        step_d2q9_kernel<S, unsigned, kUnit><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
+                                                                 (T*)gout, geo, c, status);
     else
-        step_d2q9_kernel<S, size_t><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
-                                                        (T*)gout, geo, c, status);
+        step_d2q9_kernel<S, size_t, kUnit><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
+                                                               (T*)gout, geo, c, status);
     return cudaGetLastError();
+}
+
+template <class S>
+static cudaError_t run(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
+                       const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
+{
+    if constexpr (has_unit_step_2d<S>::value) {
+        if (unit_rates_2d(hc)) return run_as<S, true>(fin, gin, fout, gout, geo, hc, status, block, st);
+    }
+    return run_as<S, false>(fin, gin, fout, gout, geo, hc, status, block, st);
 }
 
 cudaError_t launch_step_d2q9(int prec, const void* fin, const void* gin, void* fout, void* gout,

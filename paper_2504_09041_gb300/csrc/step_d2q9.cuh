@@ -24,7 +24,7 @@ using Coeffs2D = Coeffs<R, 9, 9>;
 // bounce-back (adiabatic) or anti-bounce-back (fixed T) for g at the walls (Sec. 6.1), in
 // deviations: the anti-bounce-back g_a = -g~_abar + 2 w_a T_w becomes
 // gamma_a = -gamma~_abar + 2 w_a (T_w - T_o).
-template <class S, class Idx = size_t>
+template <class S, class Idx = size_t, bool kRaw = false>
 __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
                                           const typename S::T* __restrict__ gin, const Geometry& geo,
                                           const NodeWalls<typename S::R>& w, int i, typename S::R T_ref,
@@ -38,15 +38,15 @@ __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
         R tw;
         const int s = link_source<e9(a, 0), e9(a, 1), 0>(geo, w, i, &out, &dir, &tw);
         const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-        f[a] = S::load_dev(fin, off, R(w9(a)));
-        const R gv = S::load_dev(gin, off, R(w9(a)) * T_ref);
-        g[a] = dir ? R(2.0 * w9(a)) * (tw - T_ref) - gv : gv;
+        f[a] = load_link<S, kRaw>(fin, off, R(w9(a)));
+        const R gv = load_link<S, kRaw>(gin, off, R(w9(a)) * T_ref);
+        g[a] = dir ? anti_bounce<S, kRaw>(gv, w9(a), tw, T_ref) : gv;
     });
 }
 
 // The same pull at a node whose eight neighbours all lie inside the box: no wall and no
 // periodic wrap touches any link, so every population comes straight from its upwind node.
-template <class S, class Idx = size_t>
+template <class S, class Idx = size_t, bool kRaw = false>
 __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restrict__ fin,
                                                    const typename S::T* __restrict__ gin,
                                                    const Geometry& geo, int i, typename S::R T_ref,
@@ -56,8 +56,8 @@ __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restri
     static_for<9>([&](auto A) {
         constexpr int a = decltype(A)::value;
         const Idx off = (Idx)a * geo.n + (i - (e9(a, 0) + e9(a, 1) * geo.nx));
-        f[a] = S::load_dev(fin, off, R(w9(a)));
-        g[a] = S::load_dev(gin, off, R(w9(a)) * T_ref);
+        f[a] = load_link<S, kRaw>(fin, off, R(w9(a)));
+        g[a] = load_link<S, kRaw>(gin, off, R(w9(a)) * T_ref);
     });
 }
 
@@ -171,36 +171,156 @@ __device__ __forceinline__ void from_central_d2q9(R p[3][3], R f[9], R ux, R uy)
     });
 }
 
-// One time step at one node: pull, macroscopic fields (App. A Step 7, App. B Step 7, Sec. 6.1
-// Boussinesq force), collide f and g, store.
+// The storage forms that have the reduced collision below.
+template <class S>
+struct has_unit_step_2d : std::integral_constant<bool, !std::is_same<S, StoreF32>::value> {};
+
+// Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
+// y (unit_rates_2d, checked by the host), from the stored numbers in f and g (load_raw).  Used for FP64
+// storage, bound by the FP64 pipe, and FP16 storage, bound by issue; FP32 storage, bound by the
+// memory, keeps the general collision and with it its rounding.
+//
+// A moment relaxed at rate 1 lands on its attractor plus half its source, so the collision needs, of the
+// flow, rho, j, the two shear moments and the few moments that the force multiplies, and, of the
+// energy, T and the first-order moments: they are taken from raw sums of the links, shifted with
+// rho u = j + F / 2 (j_x = rho u_x without a force along x).  The relaxed central moments are held as
+// deviations e from the rest state moving at u (1, 1/3 on 20 and 02, 1/9 on 22, times kUnits for the
+// flow and T_o for the energy), whose share of the inverse sweeps is the rest weights; so, as in the
+// general form, no O(1) number is rounded on the way to the stored one.
 template <class S, class Idx>
-__device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__ fin,
-                                               const typename S::T* __restrict__ gin,
-                                               typename S::T* __restrict__ fout,
-                                               typename S::T* __restrict__ gout, const Geometry& geo,
-                                               const Coeffs2D<typename S::R>& c, unsigned* status,
-                                               int x, int y)
+__device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9], const typename S::R g[9],
+                                                        typename S::T* __restrict__ fout,
+                                                        typename S::T* __restrict__ gout,
+                                                        const Geometry& geo,
+                                                        const UnitCoeffs<typename S::R>& c,
+                                                        unsigned* status, int i)
 {
     using R = typename S::R;
-    const int i = x + geo.nx * y;
-    R f[9], g[9];
-    // Which pull: decided per warp where possible, so that a warp holding an x-wall node of an
-    // interior row runs one x-only pull instead of both the interior and the general pull.
-    const bool y_in = y > 0 && y < geo.ny - 1;
-    const bool in = y_in && x > 0 && x < geo.nx - 1;
-    const unsigned lanes = __activemask();
-    if (__all_sync(lanes, in)) {
-        pull_d2q9_interior<S, Idx>(fin, gin, geo, i, c.T_ref, f, g);
-    } else if (__all_sync(lanes, y_in)) {
-        const NodeWalls<R> w = node_walls_x<R>(geo, x, y, 0);
-        pull_d2q9<S, Idx>(fin, gin, geo, w, i, c.T_ref, f, g);
-    } else if (in) {
-        pull_d2q9_interior<S, Idx>(fin, gin, geo, i, c.T_ref, f, g);
-    } else {
-        const NodeWalls<R> w = node_walls<R>(geo, x, y, 0, 2);
-        pull_d2q9<S, Idx>(fin, gin, geo, w, i, c.T_ref, f, g);
+    constexpr double kS = S::kUnits;
+    const R third = R(1.0 / 3.0), half = R(0.5);
+    // raw sums of the flow, rows e_y = -1, 0, 1: (7, 4, 8), (3, 0, 1), (6, 2, 5).  For stored
+    // populations the rest weights come off exactly: (a - 2 w) + c has no rounding.
+    R k0[3], d[3], s[3];
+    {
+        constexpr int row[3][3] = {{7, 4, 8}, {3, 0, 1}, {6, 2, 5}};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const R a = f[row[j][0]], b = f[row[j][1]], cc = f[row[j][2]];
+            d[j] = cc - a;
+            if constexpr (S::kFull) {
+                s[j] = (a - R(2.0 * w9(row[j][0]))) + cc;
+                k0[j] = s[j] + (b - R(w9(row[j][1])));
+            } else {
+                s[j] = a + cc;
+                k0[j] = s[j] + b;
+            }
+        }
+    }
+    const R Myy = k0[0] + k0[2], drho = Myy + k0[1];
+    const R jx = (d[0] + d[2]) + d[1], jy = k0[2] - k0[0];
+    const R Mxx = (s[0] + s[2]) + s[1], Mxy = d[2] - d[0], Mxxy = s[2] - s[0];
+    // raw sums of the energy
+    const R T0 = S::kFull ? c.T_ref : R(kS) * c.T_ref;
+    const R top = g[2] + (g[5] + g[6]), bot = g[4] + (g[7] + g[8]);
+    const R g0 = S::kFull ? g[0] - T0 : g[0];
+    const R dT = (g0 + (g[1] + g[3])) + (top + bot);
+    const R jgy = top - bot;
+    const R jgx = (g[1] - g[3]) + ((g[5] - g[6]) + (g[8] - g[7]));
+    const R T = T0 + dT, rho = R(kS) + drho;
+    check_node_bits(status, rho, T);
+
+    const R irho = recip(rho);
+    const R Fy = c.gbeta * dT, hF = half * Fy;
+    const R py = jy + hF;                        // rho u_y
+    const R ux = jx * irho, uy = py * irho;
+    const R uxh = half * ux, uyh = half * uy;
+
+    R p[3][3];   // [y link][x moment]: x moments of order 1, 2 halved
+    {
+        // pre-collision central moments of order 2 (e20, e02: less kS / 3) and kappa_21
+        const R k11 = (Mxy - jx * uy) + hF * ux;
+        const R e20p = Mxx - jx * ux;
+        const R e02p = Myy - (py - Fy) * uy;
+        const R k20 = R(kS / 3.0) + e20p;
+        const R k21 = (Mxxy - uy * k20) - ux * (k11 + Mxy);
+        // relaxation and sources (sigma_21 = F_y kappa_20 / rho, sigma_12 = 2 F_y kappa_11 / rho,
+        // sigma_22 = 2 F_y kappa_21 / rho), moments of order 1-2 per axis halved per axis
+        const R G = Fy * irho;
+        const R td = c.kf[0] * (e20p - e02p);
+        const R a3 = third * drho;
+        const R e20 = a3 + half * td, e02 = a3 - half * td;
+        const R t11 = c.kf[1] * k11;
+        const R q11 = R(0.25) * t11;
+        const R G4 = R(0.25) * G;
+        const R q12 = G4 * k11;
+        const R h21 = G4 * k20;                 // t21 / 2 = G k20 / 4
+        const R e22 = (R(kS / 9.0) * drho + e20 * e02 + (t11 + t11) * t11) * irho + G * k21;
+        // y sweep; x moment 0: (kS + drho, F/2, kS/3 + e02)
+        {
+            const R h1 = half * hF, r1 = half * (py + hF);
+            const R r2 = half * e02 + uy * (h1 + r1);
+            p[0][0] = r2 - r1;
+            p[1][0] = drho - R(2) * r2;
+            p[2][0] = r2 + r1;
+        }
+        unline0(q11, q12, uy + uy, p[0][1], p[1][1], p[2][1]);
+        {   // x moment 2, halved: (kS/6 + e20/2, t21/2, kS/18 + e22/2), orders 1-2 in y halved again
+            const R e20h = half * e20;
+            unline(e20h, R(kS / 6.0) + e20h, half * h21, R(0.25) * e22, uy, uyh, p[0][2], p[1][2], p[2][2]);
+        }
+    }
+    R df[9], dg[9];
+    unline(p[0][0], R(kS / 6.0) + p[0][0], p[0][1], p[0][2], ux, uxh, df[7], df[4], df[8]);
+    unline(p[1][0], R(kS * 2.0 / 3.0) + p[1][0], p[1][1], p[1][2], ux, uxh, df[3], df[0], df[1]);
+    unline(p[2][0], R(kS / 6.0) + p[2][0], p[2][1], p[2][2], ux, uxh, df[6], df[2], df[5]);
+
+    // energy: T, (1 - omega) eta_1, then c_s^2 T, (2/3) c_s^2 t_1 and c_s^4 T
+    {
+        const R t10 = c.kg[0] * (jgx - ux * T);
+        const R t01 = c.kg[1] * (jgy - uy * T);
+        const R T6 = R(1.0 / 6.0) * T, dT6 = R(1.0 / 6.0) * dT;
+        unline(dT, T, half * t01, dT6, uy, uyh, p[0][0], p[1][0], p[2][0]);
+        {   // x moment 1, halved: (t10, 0, (2/9) t10) / 2
+            const R h = half * t10;
+            const R r1 = uyh * h, r2 = R(1.0 / 9.0) * h + uy * r1;
+            p[0][1] = r2 - r1;
+            p[1][1] = h - R(2) * r2;
+            p[2][1] = r2 + r1;
+        }
+        unline(dT6, T6, R(1.0 / 18.0) * t01, R(1.0 / 36.0) * dT, uy, uyh, p[0][2], p[1][2], p[2][2]);
+        const R c6 = S::kFull ? c.T_ref6 : R(kS) * c.T_ref6, c23 = S::kFull ? c.T_ref23 : R(kS) * c.T_ref23;
+        unline(p[0][0], c6 + p[0][0], p[0][1], p[0][2], ux, uxh, dg[7], dg[4], dg[8]);
+        unline(p[1][0], c23 + p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
+        unline(p[2][0], c6 + p[2][0], p[2][1], p[2][2], ux, uxh, dg[6], dg[2], dg[5]);
     }
 
+    if constexpr (std::is_same<S, StoreF16S>::value) {
+        if (c.fp16_sr) {
+            store_node_f16s_sr<9, 9, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg);
+        } else {
+            static_for<9>([&](auto A) {
+                constexpr int a = decltype(A)::value;
+                StoreF16S::store_scaled(fout, (Idx)a * geo.n + i, df[a]);
+                StoreF16S::store_scaled(gout, (Idx)a * geo.n + i, dg[a]);
+            });
+        }
+    } else {
+        static_for<9>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            S::store_dev(fout, (Idx)a * geo.n + i, df[a], R(w9(a)));
+            S::store_dev(gout, (Idx)a * geo.n + i, dg[a], c.wT[a == 0 ? 0 : (a < 5 ? 1 : 2)]);
+        });
+    }
+}
+
+// Macroscopic fields, both collisions and the store of one node at any rates, from the pulled deviations.
+template <class S, class Idx>
+__device__ __forceinline__ void collide_store_d2q9(typename S::R f[9], typename S::R g[9],
+                                                   typename S::T* __restrict__ fout,
+                                                   typename S::T* __restrict__ gout, const Geometry& geo,
+                                                   const Coeffs2D<typename S::R>& c, unsigned* status, int i)
+{
+    using R = typename S::R;
     // rho = 1 + sum delta, rho u = sum delta e + F/2, T = T_o + sum gamma (sum w = 1, sum w e = 0)
     const R dT = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
     const R drho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
@@ -248,16 +368,55 @@ __device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__
     });
 }
 
-template <class S, class Idx>
+template <class S, bool kUnit>
+using StepCoeffs2D = typename std::conditional<kUnit, UnitCoeffs<typename S::R>, Coeffs2D<typename S::R>>::type;
+
+// One time step at one node: pull, macroscopic fields (App. A Step 7, App. B Step 7, Sec. 6.1
+// Boussinesq force), collide f and g, store.  kUnit: the reduced collision above.
+template <class S, class Idx, bool kUnit = false>
+__device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__ fin,
+                                               const typename S::T* __restrict__ gin,
+                                               typename S::T* __restrict__ fout,
+                                               typename S::T* __restrict__ gout, const Geometry& geo,
+                                               const StepCoeffs2D<S, kUnit>& c, unsigned* status,
+                                               int x, int y)
+{
+    using R = typename S::R;
+    const int i = x + geo.nx * y;
+    R f[9], g[9];
+    // Which pull: decided per warp where possible, so that a warp holding an x-wall node of an
+    // interior row runs one x-only pull instead of both the interior and the general pull.
+    const bool y_in = y > 0 && y < geo.ny - 1;
+    const bool in = y_in && x > 0 && x < geo.nx - 1;
+    const unsigned lanes = __activemask();
+    if (__all_sync(lanes, in)) {
+        pull_d2q9_interior<S, Idx, kUnit>(fin, gin, geo, i, c.T_ref, f, g);
+    } else if (__all_sync(lanes, y_in)) {
+        const NodeWalls<R> w = node_walls_x<R>(geo, x, y, 0);
+        pull_d2q9<S, Idx, kUnit>(fin, gin, geo, w, i, c.T_ref, f, g);
+    } else if (in) {
+        pull_d2q9_interior<S, Idx, kUnit>(fin, gin, geo, i, c.T_ref, f, g);
+    } else {
+        const NodeWalls<R> w = node_walls<R>(geo, x, y, 0, 2);
+        pull_d2q9<S, Idx, kUnit>(fin, gin, geo, w, i, c.T_ref, f, g);
+    }
+
+    if constexpr (kUnit) {
+        collide_store_d2q9_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
+    } else {
+        collide_store_d2q9<S, Idx>(f, g, fout, gout, geo, c, status, i);
+    }
+}
+template <class S, class Idx, bool kUnit = false>
 __global__ void __launch_bounds__(256)
     step_d2q9_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                      typename S::T* __restrict__ fout, typename S::T* __restrict__ gout, Geometry geo,
-                     Coeffs2D<typename S::R> c, unsigned* status)
+                     StepCoeffs2D<S, kUnit> c, unsigned* status)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= geo.nx || y >= geo.ny) return;
-    node_step_d2q9<S, Idx>(fin, gin, fout, gout, geo, c, status, x, y);
+    node_step_d2q9<S, Idx, kUnit>(fin, gin, fout, gout, geo, c, status, x, y);
 }
 
 }  // namespace lbm
