@@ -26,7 +26,7 @@
 namespace lbm {
 
 // What the reduced step needs of a member, for the storage forms that have one.
-template <class S, bool = has_unit_step_2d<S>::value>
+template <class S, bool = has_unit_step<S>::value>
 struct BatchUnit {
     UnitCoeffs<typename S::R> u;
     int unit;                 // the member takes the reduced collision (unit_rates_2d)
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(256, BatchBounds<S>::kMinBlocks)
         const int x = (local % m.tiles_x) * tile_x + (int)threadIdx.x % tile_x;
         const int y = (local / m.tiles_x) * tile_y + (int)threadIdx.x / tile_x;
         if (x >= m.geo.nx || y >= m.geo.ny) continue;
-        if constexpr (has_unit_step_2d<S>::value) {
+        if constexpr (has_unit_step<S>::value) {
             if (m.unit) {
                 node_step_d2q9<S, unsigned, true>(fin + m.off, gin + m.off, fout + m.off, gout + m.off,
                                                   m.geo, m.u, status + k, x, y);
@@ -206,7 +206,7 @@ std::vector<lbm::BatchMember<S>> member_table(const lbm_batch_s* b)
         t[k].off = b->off[k];
         t[k].tile0 = tile;
         t[k].tiles_x = (P.nx + b->tile_x - 1) / b->tile_x;
-        if constexpr (lbm::has_unit_step_2d<S>::value) {
+        if constexpr (lbm::has_unit_step<S>::value) {
             t[k].u = lbm::make_unit_coeffs<R, 2>(P.hc);
             t[k].unit = lbm::unit_rates_2d(P.hc) ? 1 : 0;
         }

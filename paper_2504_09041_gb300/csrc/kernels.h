@@ -161,6 +161,14 @@ inline UnitCoeffs<R> make_unit_coeffs(const HostCoeffs& h)
     return c;
 }
 
+// The coefficients of the 3D step's collision instance kU.
+template <class R, int kU>
+inline auto make_step_coeffs(const HostCoeffs& h)
+{
+    if constexpr (kU == 3) return make_unit_coeffs<R, 3>(h);
+    else return make_coeffs<R, 27, 15>(h);
+}
+
 // Default thread blocks, x-major so that a warp reads and writes 32 consecutive nodes; a
 // caller-chosen shape (block.x > 0) replaces it.  2D: 256 threads.  3D: 64 x 1, which at 96
 // registers per thread lets 10 blocks (20 warps) share an SM against 16 warps for 256-thread
@@ -216,11 +224,13 @@ inline bool unit_rates_2d(const HostCoeffs& h)
 }
 
 // Which collision instance the 3D step takes: 0 general, 1 unit-rate energy collision, 2 that and
-// the unit-rate flow relaxation.
+// the unit-rate flow relaxation, 3 that with gravity along z (collide_store_d3q27_unit; FP32 storage
+// takes instance 2 there, see has_unit_step).
 inline int rate_class(const HostCoeffs& h)
 {
     if (!unit_energy_rates(h)) return 0;
-    return unit_flow_rates(h) ? 2 : 1;
+    if (!unit_flow_rates(h)) return 1;
+    return h.gaxis == 2 ? 3 : 2;
 }
 
 // Rows per thread of the 3D FP32 / FP16S step: the handle's setting, or when that is 0 the faster
@@ -230,7 +240,7 @@ inline int rate_class(const HostCoeffs& h)
 inline int rows3d_for(const HostCoeffs& h, bool f16s)
 {
     if (h.rows3d > 0) return h.rows3d;
-    return f16s && rate_class(h) == 2 ? 1 : 2;
+    return f16s && rate_class(h) >= 2 ? 1 : 2;
 }
 
 inline dim3 grid_shape(const Geometry& g, dim3 b)

@@ -25,7 +25,7 @@ enum FaceKind { kPeriodic = 0, kAdiabatic = 1, kFixedT = 2 };
 //    normal range (full 11-bit significand) while |deviation| < 64 still fits; the scale is a
 //    power of two and adds no rounding.
 //
-// The reduced steps (default rates and gravity axis) take the stored number itself (load_raw) and
+// The reduced steps (default rates and gravity axis; FP64 and F16S) take the stored number itself (load_raw) and
 // work in its units: every relation of the step is homogeneous of degree one in the populations, so
 // multiplying them all by kUnits only multiplies the rest state's constants.  kFull: the stored
 // number is the population, not its deviation; the rest state is then taken off in the raw sums.
@@ -57,9 +57,6 @@ __device__ __forceinline__ __half ldg_pf256(const __half* p)
 struct StoreF32 {
     using T = float;
     using R = float;
-    static constexpr bool kFull = false;
-    static constexpr double kUnits = 1.0;
-    __device__ static R load_raw(const T* p, size_t i) { return ldg_pf256(p + i); }
     __device__ static R load_dev(const T* p, size_t i, R) { return ldg_pf256(p + i); }
     __device__ static void store_dev(T* p, size_t i, R dev, R) { p[i] = dev; }
 };
@@ -125,6 +122,11 @@ __device__ __forceinline__ unsigned sr_pair_bits(unsigned seed)
     return seed * mult;
 }
 
+
+// The storage forms that have reduced steps: FP64, bound by the FP64 pipe, and FP16, bound by issue.
+// FP32 storage is bound by the memory and keeps the general collisions with their rounding.
+template <class S>
+struct has_unit_step : std::integral_constant<bool, !std::is_same<S, StoreF32>::value> {};
 
 // Box geometry and wall description shared by every kernel.
 struct Geometry {
@@ -293,30 +295,37 @@ __device__ __forceinline__ typename S::R anti_bounce(typename S::R gv, double w,
                                                      typename S::R T_ref)
 {
     using R = typename S::R;
-    if constexpr (kRaw && S::kFull) return R(2.0 * w) * tw - gv;
-    else if constexpr (kRaw) return R(2.0 * S::kUnits * w) * (tw - T_ref) - gv;
-    else return R(2.0 * w) * (tw - T_ref) - gv;
+    if constexpr (kRaw) {
+        if constexpr (S::kFull) return R(2.0 * w) * tw - gv;
+        else return R(2.0 * S::kUnits * w) * (tw - T_ref) - gv;
+    } else {
+        return R(2.0 * w) * (tw - T_ref) - gv;
+    }
 }
+
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 
 // One line of an inverse sweep whose moments of order 1 and 2 come in halved (h1, h2) and whose
 // order-0 moment is split into a constant and the rest k0: (k0 + const, 2 h1, 2 h2 + const / 3) at
 // velocity u -> the deviations of the three links from the constant's rest weights.  k0f is the full
 // order-0 moment and uh = u / 2.  Six operations; the halvings of uncentral_line are carried by the
-// inputs instead (exact: powers of two).
+// inputs instead (exact: powers of two).  The fused operations are written out: from k0 - 2 r2 the
+// compiler makes two additions.
 template <class R>
 __device__ __forceinline__ void unline(R k0, R k0f, R h1, R h2, R u, R uh, R& a, R& b, R& c)
 {
-    const R r1 = h1 + uh * k0f;           // half the raw first moment
-    const R r2 = h2 + u * (h1 + r1);      // half the raw second moment (deviation)
+    const R r1 = fma_(uh, k0f, h1);          // half the raw first moment
+    const R r2 = fma_(u, h1 + r1, h2);       // half the raw second moment (deviation)
     a = r2 - r1;
-    b = k0 - R(2) * r2;
+    b = fma_(R(-2), r2, k0);
     c = r2 + r1;
 }
 // The same with a zero order-0 moment; u2 = 2 u.
 template <class R>
 __device__ __forceinline__ void unline0(R h1, R h2, R u2, R& a, R& b, R& c)
 {
-    const R r2 = h2 + u2 * h1;
+    const R r2 = fma_(u2, h1, h2);
     a = r2 - h1;
     b = R(-2) * r2;
     c = r2 + h1;

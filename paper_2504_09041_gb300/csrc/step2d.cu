@@ -28,7 +28,7 @@ template <class S>
 static cudaError_t run(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
                        const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
 {
-    if constexpr (has_unit_step_2d<S>::value) {
+    if constexpr (has_unit_step<S>::value) {
         if (unit_rates_2d(hc)) return run_as<S, true>(fin, gin, fout, gout, geo, hc, status, block, st);
     }
     return run_as<S, false>(fin, gin, fout, gout, geo, hc, status, block, st);

@@ -7,8 +7,7 @@
 
 namespace lbm {
 
-// kU: the collision instance for the rates (rate_class: 0 general, 1 unit-rate energy collision,
-// 2 unit-rate energy collision and flow relaxation).
+// kU: the collision instance for the rates (rate_class).
 template <int kU>
 static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
@@ -18,7 +17,7 @@ static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fou
     using T = typename S::T;
     using R = typename S::R;
     const dim3 b = block_shape(geo.nx, block, 3);
-    const auto c = make_coeffs<R, 27, 15>(hc);
+    const auto c = make_step_coeffs<R, kU>(hc);
     const int rows = rows3d_for(hc, true);
     if (step_index32(geo, 27, hc) && rows == 2) {
         dim3 g = grid_shape(geo, b);
@@ -44,6 +43,7 @@ cudaError_t launch_step_d3q27_f16s(const void* fin, const void* gin, void* fout,
                                   dim3 block, cudaStream_t st)
 {
     switch (rate_class(hc)) {
+    case 3: return launch_plain_f16s<3>(fin, gin, fout, gout, geo, hc, status, block, st);
     case 2: return launch_plain_f16s<2>(fin, gin, fout, gout, geo, hc, status, block, st);
     case 1: return launch_plain_f16s<1>(fin, gin, fout, gout, geo, hc, status, block, st);
     }
@@ -59,7 +59,7 @@ static cudaError_t launch_tma_f16s(const TmaMaps& tm, const void* fin, const voi
     using T = typename S::T;
     using R = typename S::R;
     using L = TmaLayout<T, TY>;
-    const auto c = make_coeffs<R, 27, 15>(hc);
+    const auto c = make_step_coeffs<R, kU>(hc);
     const int tiles_x = (geo.nx + kTmaTX - 1) / kTmaTX, tiles_y = (geo.ny + TY - 1) / TY;
     const int n_tiles = tiles_x * tiles_y * geo.nz;
     const dim3 block(kTmaTX * TY + 32, 1, 1);   // TY rows of consumers and one producer warp
@@ -96,6 +96,7 @@ cudaError_t launch_step_d3q27_tma_f16s(const TmaMaps& tm, const void* fin, const
                                       unsigned* status, cudaStream_t st)
 {
     switch (rate_class(hc)) {
+    case 3: return launch_tma_rows_f16s<3>(tm, fin, gin, fout, gout, geo, hc, status, st);
     case 2: return launch_tma_rows_f16s<2>(tm, fin, gin, fout, gout, geo, hc, status, st);
     case 1: return launch_tma_rows_f16s<1>(tm, fin, gin, fout, gout, geo, hc, status, st);
     }

@@ -5,8 +5,7 @@
 
 namespace lbm {
 
-// kU: the collision instance for the rates (rate_class: 0 general, 1 unit-rate energy collision,
-// 2 unit-rate energy collision and flow relaxation).
+// kU: the collision instance for the rates (rate_class).
 template <int kU>
 static cudaError_t launch_plain_f64(const void* fin, const void* gin, void* fout, void* gout,
                                     const Geometry& geo, const HostCoeffs& hc, unsigned* status,
@@ -16,7 +15,7 @@ static cudaError_t launch_plain_f64(const void* fin, const void* gin, void* fout
     using T = typename S::T;
     using R = typename S::R;
     const dim3 b = block_shape(geo.nx, block, 3);
-    const auto c = make_coeffs<R, 27, 15>(hc);
+    const auto c = make_step_coeffs<R, kU>(hc);
     if (step_index32(geo, 27, hc))
         step_d3q27_kernel<S, unsigned, 1, kU><<<grid_shape(geo, b), b, 0, st>>>(
             (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
@@ -31,6 +30,7 @@ cudaError_t launch_step_d3q27_f64(const void* fin, const void* gin, void* fout, 
                                   dim3 block, cudaStream_t st)
 {
     switch (rate_class(hc)) {
+    case 3: return launch_plain_f64<3>(fin, gin, fout, gout, geo, hc, status, block, st);
     case 2: return launch_plain_f64<2>(fin, gin, fout, gout, geo, hc, status, block, st);
     case 1: return launch_plain_f64<1>(fin, gin, fout, gout, geo, hc, status, block, st);
     }

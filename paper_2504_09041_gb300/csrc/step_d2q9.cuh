@@ -171,10 +171,6 @@ __device__ __forceinline__ void from_central_d2q9(R p[3][3], R f[9], R ux, R uy)
     });
 }
 
-// The storage forms that have the reduced collision below.
-template <class S>
-struct has_unit_step_2d : std::integral_constant<bool, !std::is_same<S, StoreF32>::value> {};
-
 // Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
 // y (unit_rates_2d, checked by the host), from the stored numbers in f and g (load_raw).  Used for FP64
 // storage, bound by the FP64 pipe, and FP16 storage, bound by issue; FP32 storage, bound by the
@@ -260,7 +256,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             const R h1 = half * hF, r1 = half * (py + hF);
             const R r2 = half * e02 + uy * (h1 + r1);
             p[0][0] = r2 - r1;
-            p[1][0] = drho - R(2) * r2;
+            p[1][0] = fma_(R(-2), r2, drho);
             p[2][0] = r2 + r1;
         }
         unline0(q11, q12, uy + uy, p[0][1], p[1][1], p[2][1]);
@@ -284,7 +280,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             const R h = half * t10;
             const R r1 = uyh * h, r2 = R(1.0 / 9.0) * h + uy * r1;
             p[0][1] = r2 - r1;
-            p[1][1] = h - R(2) * r2;
+            p[1][1] = fma_(R(-2), r2, h);
             p[2][1] = r2 + r1;
         }
         unline(dT6, T6, R(1.0 / 18.0) * t01, R(1.0 / 36.0) * dT, uy, uyh, p[0][2], p[1][2], p[2][2]);

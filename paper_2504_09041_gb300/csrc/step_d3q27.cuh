@@ -33,7 +33,7 @@ __host__ __device__ constexpr int g15_of_27(int a)
     return a < 7 ? a : (a >= 19 ? a - 12 : -1);
 }
 
-template <class S, class Idx = size_t>
+template <class S, class Idx = size_t, bool kRaw = false>
 __device__ __forceinline__ void pull_d3q27_d3q15(const typename S::T* __restrict__ fin,
                                                  const typename S::T* __restrict__ gin,
                                                  const Geometry& geo,
@@ -49,19 +49,19 @@ __device__ __forceinline__ void pull_d3q27_d3q15(const typename S::T* __restrict
         R tw;
         const int s = link_source<e27(a, 0), e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
         const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-        f[a] = S::load_dev(fin, off, R(w27(a)));
+        f[a] = load_link<S, kRaw>(fin, off, R(w27(a)));
         constexpr int b = g15_of_27(a);
         if constexpr (b >= 0) {
             constexpr int ob = opp15(b);
             const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
-            const R gv = S::load_dev(gin, og, R(w15(b)) * T_ref);
-            g[b] = dir ? R(2.0 * w15(b)) * (tw - T_ref) - gv : gv;
+            const R gv = load_link<S, kRaw>(gin, og, R(w15(b)) * T_ref);
+            g[b] = dir ? anti_bounce<S, kRaw>(gv, w15(b), tw, T_ref) : gv;
         }
     });
 }
 
 // The same pull at a node whose 26 neighbours all lie inside the box (no wall, no wrap).
-template <class S, class Idx = size_t>
+template <class S, class Idx = size_t, bool kRaw = false>
 __device__ __forceinline__ void pull_d3q27_d3q15_interior(const typename S::T* __restrict__ fin,
                                                           const typename S::T* __restrict__ gin,
                                                           const Geometry& geo, int i,
@@ -72,9 +72,9 @@ __device__ __forceinline__ void pull_d3q27_d3q15_interior(const typename S::T* _
     static_for<27>([&](auto A) {
         constexpr int a = decltype(A)::value;
         const int s = i - (e27(a, 0) + e27(a, 1) * geo.nx + e27(a, 2) * geo.nxy);
-        f[a] = S::load_dev(fin, (Idx)a * geo.n + s, R(w27(a)));
+        f[a] = load_link<S, kRaw>(fin, (Idx)((Idx)a * geo.n + s), R(w27(a)));
         constexpr int b = g15_of_27(a);
-        if constexpr (b >= 0) g[b] = S::load_dev(gin, (Idx)b * geo.n + s, R(w15(b)) * T_ref);
+        if constexpr (b >= 0) g[b] = load_link<S, kRaw>(gin, (Idx)((Idx)b * geo.n + s), R(w15(b)) * T_ref);
     });
 }
 
@@ -572,10 +572,243 @@ __device__ __forceinline__ void raw01_g_d3q15(const R g[15], R& r000, R& r100, R
     r001 = (g[5] - g[6]) + Cz;
 }
 
+// Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
+// z (rate_class 3, checked by the host), from the stored numbers in f and g (load_raw); the 3D
+// counterpart of collide_store_d2q9_unit, see there.  Of the flow's moments only those enter that
+// relax with a rate of their own (rho, j and order 2) or that the force multiplies (orders 0-1 in z, up
+// to 2 in x and y); t_210 and t_120 vanish.  The relaxed moments are held as deviations e from the
+// rest state moving at u (1, 1/3, 1/9, 1/27 on the moments even in every direction, times kUnits) and
+// halved once per axis of non-zero order, as the inverse sweeps want them.  About 595 FP64 instructions
+// per node against 867 with the two reduced collisions above alone: 128^3 in FP64 2.33 ms against
+// 3.36 per step; FP16 storage issues 1,012 instructions against 1,249: 81 us against 95 at 128^3, where
+// half of it comes from L2.
+template <class S, class Idx>
+__device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[27], const typename S::R g[15],
+                                                         typename S::T* __restrict__ fout,
+                                                         typename S::T* __restrict__ gout,
+                                                         const Geometry& geo,
+                                                         const UnitCoeffs<typename S::R>& c,
+                                                         unsigned* status, int i)
+{
+    using R = typename S::R;
+    constexpr double kS = S::kUnits;
+    const R third = R(1.0 / 3.0), half = R(0.5), quarter = R(0.25), two = R(2);
+
+    // raw moments: m[k][b][a] = sum e_x^a e_y^b over layer k (e_z = k - 1)
+    R m[3][3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        R q[3][3];   // [j][a]
+        static_for<3>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            // (the links of a layer's lines; k is unrolled, so the indices fold)
+            const int la = k == 0 ? idx27(-1, j - 1, -1) : (k == 1 ? idx27(-1, j - 1, 0) : idx27(-1, j - 1, 1));
+            const int lb = k == 0 ? idx27(0, j - 1, -1) : (k == 1 ? idx27(0, j - 1, 0) : idx27(0, j - 1, 1));
+            const int lc = k == 0 ? idx27(1, j - 1, -1) : (k == 1 ? idx27(1, j - 1, 0) : idx27(1, j - 1, 1));
+            const R a = f[la], b = f[lb], cc = f[lc];
+            q[j][1] = cc - a;
+            if constexpr (S::kFull) {   // the rest weights come off exactly
+                q[j][2] = (a - R(2.0 * w27(la))) + cc;
+                q[j][0] = q[j][2] + (b - R(w27(lb)));
+            } else {
+                q[j][2] = a + cc;
+                q[j][0] = q[j][2] + b;
+            }
+        });
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            m[k][2][a] = q[0][a] + q[2][a];
+            m[k][1][a] = q[2][a] - q[0][a];
+            m[k][0][a] = m[k][2][a] + q[1][a];
+        }
+    }
+    R z0[3][3], z1[3][3];   // [b][a]: orders 0 and 1 in z
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            z0[b][a] = (m[0][b][a] + m[2][b][a]) + m[1][b][a];
+            z1[b][a] = m[2][b][a] - m[0][b][a];
+        }
+    const R M002 = m[0][0][0] + m[2][0][0];
+    const R drho = z0[0][0], jx = z0[0][1], jy = z0[1][0], jz = z1[0][0];
+
+    // energy: T and the first-order moments
+    const R T0 = S::kFull ? c.T_ref : R(kS) * c.T_ref;
+    R dT, gx, gy, gz;
+    {
+        R gs[15];
+#pragma unroll
+        for (int b = 0; b < 15; ++b) gs[b] = g[b];
+        if constexpr (S::kFull) gs[0] -= T0;
+        raw01_g_d3q15(gs, dT, gx, gy, gz);
+    }
+    const R T = T0 + dT, rho = R(kS) + drho;
+    check_node_bits(status, rho, T);
+    const R irho = recip(rho);
+    const R Fz = c.gbeta * dT, hF = half * Fz;
+    const R pz = jz + hF;                                  // rho u_z (u_x, u_y: no force)
+    const R ux = jx * irho, uy = jy * irho, uz = pz * irho;
+    const R uxh = half * ux, uyh = half * uy, uzh = half * uz;
+
+    R p[3][3][3];   // z links, then orders in y and x (halved per axis of non-zero order)
+    {
+        // pre-collision central moments
+        const R k110 = z0[1][1] - ux * jy;
+        const R k101 = z1[0][1] - ux * jz;
+        const R k011 = z1[1][0] - uy * jz;
+        const R E200 = z0[0][2] - ux * jx, E020 = z0[2][0] - uy * jy, E002 = M002 - uz * (jz - hF);
+        const R k200 = R(kS / 3.0) + E200, k020 = R(kS / 3.0) + E020;
+        const R a21 = z0[1][2] - ux * (z0[1][1] + k110);                  // (e_x - u_x)^2 e_y
+        const R m020 = R(kS / 3.0) + z0[2][0];
+        const R a12 = z0[2][1] - ux * m020;                               // (e_x - u_x) e_y^2
+        const R a22 = (R(kS / 9.0) + z0[2][2]) - ux * (z0[2][1] + a12);
+        const R k120 = a12 - uy * (k110 + k110);
+        const R k210 = a21 - uy * k200;
+        const R k220 = a22 - uy * (a21 + k210);
+        const R b20 = z1[0][2] - ux * (z1[0][1] + k101);                  // times e_z
+        const R b11 = z1[1][1] - ux * z1[1][0];
+        const R b21 = z1[1][2] - ux * (z1[1][1] + b11);
+        const R b12 = z1[2][1] - ux * z1[2][0];
+        const R b22 = z1[2][2] - ux * (z1[2][1] + b12);
+        const R c02 = z1[2][0] - uy * (z1[1][0] + k011);
+        const R c11 = b11 - uy * k101;
+        const R c12 = b12 - uy * (b11 + c11);
+        const R c21 = b21 - uy * b20;
+        const R c22 = b22 - uy * (b21 + c21);
+        const R k201 = b20 - uz * k200, k021 = c02 - uz * k020, k111 = c11 - uz * k110;
+        const R k211 = c21 - uz * k210, k121 = c12 - uz * k120, k221 = c22 - uz * k220;
+
+        // relaxation; x_abc = t_abc halved per axis of non-zero order
+        const R G = Fz * irho, G4 = quarter * G, G8 = half * G4, G16 = half * G8;
+        const R i4 = quarter * irho, i8 = half * i4, f5 = R(0.2) * irho, i6 = R(1.0 / 6.0) * irho;
+        const R t110 = c.kf[0] * k110, t101 = c.kf[1] * k101, t011 = c.kf[2] * k011;
+        const R td1 = c.kf[4] * (E200 - E020), td2 = c.kf[5] * (E200 - E002);
+        const R e200 = third * (drho + td1 + td2), e020 = e200 - td1, e002 = e200 - td2;
+        const R q200 = R(kS / 3.0) + e200, q020 = R(kS / 3.0) + e020, q002 = R(kS / 3.0) + e002;
+        const R d110 = t110 + t110, d101 = t101 + t101, d011 = t011 + t011;
+        const R x102 = G4 * k101, x012 = G4 * k011, x201 = G8 * k200, x021 = G8 * k020;
+        const R y111 = G4 * k110, x111 = quarter * y111;
+        const R l0 = R(kS * 2.0 / 9.0) * drho;
+        const R x220 = i4 * (l0 - R(kS / 3.0) * e002 + e200 * e020 + d110 * t110);
+        const R x202 = i4 * (l0 - R(kS / 3.0) * e020 + e200 * e002 + d101 * t101) + G4 * k201;
+        const R x022 = i4 * (l0 - R(kS / 3.0) * e200 + e020 * e002 + d011 * t011) + G4 * k021;
+        const R x211 = i8 * (q200 * t011 + d110 * t101) + G16 * k210;
+        const R x121 = i8 * (q020 * t101 + d110 * t011) + G16 * k120;
+        const R x112 = i8 * (q002 * t110 + d011 * t101) + G8 * k111;
+        const R x122 = f5 * (q020 * x102 + d101 * x021 + d110 * x012 + d011 * y111) + G8 * k121;
+        const R x212 = f5 * (q200 * x012 + d011 * x201 + d110 * x102 + d101 * y111) + G8 * k211;
+        const R x221 = f5 * (q200 * x021 + q020 * x201 + d110 * y111) + G16 * k220;
+        const R x222 = i6 * (q200 * x022 + q020 * x202 + q002 * x220
+                             + R(4) * (d110 * x112 + d101 * x121 + d011 * x211)) + G8 * k221;
+
+        // inverse sweep along z
+        const R uz2 = uz + uz;
+        unline(drho, rho, half * hF, half * e002, uz, uzh, p[0][0][0], p[1][0][0], p[2][0][0]);
+        unline0(quarter * t101, x102, uz2, p[0][0][1], p[1][0][1], p[2][0][1]);
+        unline0(quarter * t011, x012, uz2, p[0][1][0], p[1][1][0], p[2][1][0]);
+        unline(half * e200, half * q200, x201, x202, uz, uzh, p[0][0][2], p[1][0][2], p[2][0][2]);
+        unline(half * e020, half * q020, x021, x022, uz, uzh, p[0][2][0], p[1][2][0], p[2][2][0]);
+        const R t110q = quarter * t110;
+        unline(t110q, t110q, x111, x112, uz, uzh, p[0][1][1], p[1][1][1], p[2][1][1]);
+        unline0(x211, x212, uz2, p[0][1][2], p[1][1][2], p[2][1][2]);
+        unline0(x121, x122, uz2, p[0][2][1], p[1][2][1], p[2][2][1]);
+        unline(x220, R(kS / 36.0) + x220, x221, x222, uz, uzh, p[0][2][2], p[1][2][2], p[2][2][2]);
+    }
+    // along y, then x; wz and wy are the rest weights of the links already formed
+    R df[27], dg[15];
+    static_for<3>([&](auto K) {
+        constexpr int k = decltype(K)::value;
+        constexpr double wz = kS * (k == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
+        unline(p[k][0][0], R(wz) + p[k][0][0], p[k][1][0], p[k][2][0], uy, uyh, p[k][0][0], p[k][1][0], p[k][2][0]);
+        unline(p[k][0][1], p[k][0][1], p[k][1][1], p[k][2][1], uy, uyh, p[k][0][1], p[k][1][1], p[k][2][1]);
+        unline(p[k][0][2], R(wz / 6.0) + p[k][0][2], p[k][1][2], p[k][2][2], uy, uyh, p[k][0][2], p[k][1][2], p[k][2][2]);
+        static_for<3>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            constexpr double wy = wz * (j == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
+            unline(p[k][j][0], R(wy) + p[k][j][0], p[k][j][1], p[k][j][2], ux, uxh, df[idx27(-1, j - 1, k - 1)],
+                   df[idx27(0, j - 1, k - 1)], df[idx27(1, j - 1, k - 1)]);
+        });
+    });
+
+    // energy: the moments of collide_g_d3q15_unit as deviations from w T_o
+    {
+        constexpr double c3 = 2.0 / 9.0;
+        const R rest2 = S::kFull ? two * c.T_ref6 : R(2.0 * kS) * c.T_ref6;
+        const R t100 = c.kg[0] * (gx - ux * T), t010 = c.kg[1] * (gy - uy * T), t001 = c.kg[2] * (gz - uz * T);
+        const R q100 = t100 + ux * T, q010 = t010 + uy * T, q001 = t001 + uz * T;
+        const R xt = ux * t001;
+        const R q110 = ux * t010 + uy * q100, q101 = xt + uz * q100, q011 = uy * t001 + uz * q010;
+        const R t2 = third * dT;
+        const R q200 = t2 + ux * (t100 + q100), q020 = t2 + uy * (t010 + q010), q002 = t2 + uz * (t001 + q001);
+        const R q020f = q020 + rest2;
+        const R q120 = t100 * (R(c3) + uy * uy) + ux * q020f;
+        const R q012 = t010 * (R(c3) + uz * uz) + uy * (q002 + rest2);
+        const R q201 = t001 * (R(c3) + ux * ux) + uz * (q200 + rest2);
+        const R q111 = uy * xt + uz * q110;
+        const R Z1 = q012 - ux * (two * q110 - ux * q010);
+        const R Z2 = R(1.0 / 9.0) * dT + uy * (two * Z1 - uy * (third * T));
+        const R q220 = Z2 + ux * (two * q120 - ux * q020f);
+        dg[0] = (dT - q200) - (q020 + q002) + two * q220;
+        const R h220 = half * q220, h120 = half * q120, h012 = half * q012, h201 = half * q201;
+        const R Sx = half * q200 - h220, Sy = half * q020 - h220, Sz = half * q002 - h220;
+        const R Dx = half * q100 - h120, Dy = half * q010 - h012, Dz = half * q001 - h201;
+        dg[1] = Sx + Dx;
+        dg[2] = Sx - Dx;
+        dg[3] = Sy + Dy;
+        dg[4] = Sy - Dy;
+        dg[5] = Sz + Dz;
+        dg[6] = Sz - Dz;
+        const R e = R(0.125);
+        const R s0 = quarter * h220, sx = quarter * h120, sy = quarter * h012, sz = quarter * h201;
+        const R sxy = e * q110, sxz = e * q101, syz = e * q011, sxyz = e * q111;
+        const R P_s = s0 + sz, M_s = s0 - sz, P_y = sy + syz, M_y = sy - syz;
+        const R P_x = sx + sxz, M_x = sx - sxz, P_xy = sxy + sxyz, M_xy = sxy - sxyz;
+        const R A0 = P_s + P_y, B0 = P_s - P_y, A1 = P_x + P_xy, B1 = P_x - P_xy;
+        const R C0 = M_s + M_y, D0 = M_s - M_y, C1 = M_x + M_xy, D1 = M_x - M_xy;
+        dg[7] = A0 + A1;
+        dg[8] = A0 - A1;
+        dg[9] = B0 + B1;
+        dg[10] = B0 - B1;
+        dg[11] = C0 + C1;
+        dg[12] = C0 - C1;
+        dg[13] = D0 + D1;
+        dg[14] = D0 - D1;
+    }
+
+    if constexpr (std::is_same<S, StoreF16S>::value) {
+        if (c.fp16_sr) {
+            store_node_f16s_sr<27, 15, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg);
+        } else {
+            static_for<27>([&](auto A) {
+                constexpr int a = decltype(A)::value;
+                StoreF16S::store_scaled(fout, (Idx)a * geo.n + i, df[a]);
+            });
+            static_for<15>([&](auto B) {
+                constexpr int b = decltype(B)::value;
+                StoreF16S::store_scaled(gout, (Idx)b * geo.n + i, dg[b]);
+            });
+        }
+    } else {
+        static_for<27>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            S::store_dev(fout, (Idx)a * geo.n + i, df[a], R(w27(a)));
+        });
+        static_for<15>([&](auto B) {
+            constexpr int b = decltype(B)::value;
+            S::store_dev(gout, (Idx)b * geo.n + i, dg[b], c.wT[b == 0 ? 0 : (b < 7 ? 1 : 2)]);
+        });
+    }
+}
+
+// The coefficients of collision instance kRates (rate_class).
+template <class S, int kRates>
+using StepCoeffs3D = typename std::conditional<kRates == 3, UnitCoeffs<typename S::R>, Coeffs3D<typename S::R>>::type;
+
 // Macroscopic fields, both collisions and the store of one node whose pulled deviations are in
 // f (flow) and g (energy); i is the node's linear index.  kRates (rate_class, checked by the host):
 // 0 general rates; 1 the energy rates of lbm_create (collide_g_d3q15_unit); 2 the flow rates of
-// lbm_create as well (relax_f_d3q27<true>).
+// lbm_create as well (relax_f_d3q27<true>).  (3, gravity along z too, is collide_store_d3q27_unit.)
 template <class S, class Idx, int kRates = 0>
 __device__ __forceinline__ void collide_store_d3q27(typename S::R f[27], typename S::R g[15],
                                                     typename S::T* __restrict__ fout,
@@ -589,7 +822,7 @@ __device__ __forceinline__ void node_step_d3q27(const typename S::T* __restrict_
                                                 const typename S::T* __restrict__ gin,
                                                 typename S::T* __restrict__ fout,
                                                 typename S::T* __restrict__ gout,
-                                                const Geometry& geo, const Coeffs3D<typename S::R>& c,
+                                                const Geometry& geo, const StepCoeffs3D<S, kRates>& c,
                                                 unsigned* status, int x, int y, int z)
 {
     using R = typename S::R;
@@ -601,17 +834,18 @@ __device__ __forceinline__ void node_step_d3q27(const typename S::T* __restrict_
     const bool in = yz_in && x > 0 && x < geo.nx - 1;
     const unsigned lanes = __activemask();
     if (__all_sync(lanes, in)) {
-        pull_d3q27_d3q15_interior<S, Idx>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
     } else if (__all_sync(lanes, yz_in)) {
         const NodeWalls<R> w = node_walls_x<R>(geo, x, y, z);
-        pull_d3q27_d3q15<S, Idx>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
     } else if (in) {
-        pull_d3q27_d3q15_interior<S, Idx>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
     } else {
         const NodeWalls<R> w = node_walls<R>(geo, x, y, z, 3);
-        pull_d3q27_d3q15<S, Idx>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
     }
-    collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);
+    if constexpr (kRates == 3) collide_store_d3q27_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
+    else collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);
 }
 
 template <class S, class Idx, int kRates>
@@ -730,7 +964,7 @@ template <class S, class Idx, int kRows = 1, int kRates = 0>
 __global__ void __maxnreg__(LBM_MAXREG3D)
     step_d3q27_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                       typename S::T* __restrict__ fout, typename S::T* __restrict__ gout,
-                      Geometry geo, Coeffs3D<typename S::R> c, unsigned* status)
+                      Geometry geo, StepCoeffs3D<S, kRates> c, unsigned* status)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * kRows;

@@ -107,17 +107,12 @@ __device__ __forceinline__ void fence_mbar_init()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// Value of a stored element as a deviation from its rest value (storage policy S).
-template <class S>
-__device__ __forceinline__ typename S::R dev_of(typename S::T v, typename S::R shift);
-template <>
-__device__ __forceinline__ double dev_of<StoreF64>(double v, double shift) { return v - shift; }
-template <>
-__device__ __forceinline__ float dev_of<StoreF32>(float v, float) { return v; }
-template <>
-__device__ __forceinline__ float dev_of<StoreF16S>(__half v, float)
+// Value of a stored element: its deviation from the rest state, or with kRaw in storage units.
+template <class S, bool kRaw>
+__device__ __forceinline__ typename S::R staged_value(typename S::T v)
 {
-    return __half2float(v) * StoreF16S::kInvScale;
+    if constexpr (std::is_same<S, StoreF16S>::value) return __half2float(v) * (kRaw ? 1.0f : S::kInvScale);
+    else return v;
 }
 
 template <class S, int TY>
@@ -138,7 +133,7 @@ __device__ __forceinline__ void tma_issue_tile(const CUtensorMap* mf, const CUte
 
 // Links of a node on an x wall (or x wrap) that leave the box through x, replaced by the wall
 // rules (or the wrapped source) from global memory; the other links keep their staged values.
-template <class S, class Idx>
+template <class S, class Idx, bool kRaw>
 __device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict__ fin,
                                                  const typename S::T* __restrict__ gin,
                                                  const Geometry& geo, int x, int y, int z, int i,
@@ -158,13 +153,13 @@ __device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict
                 R tw;
                 const int s = link_source<ex, e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
                 const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-                f[a] = S::load_dev(fin, off, R(w27(a)));
+                f[a] = load_link<S, kRaw>(fin, off, R(w27(a)));
                 constexpr int b = g15_of_27(a);
                 if constexpr (b >= 0) {
                     constexpr int ob = opp15(b);
                     const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
-                    const R gv = S::load_dev(gin, og, R(w15(b)) * T_ref);
-                    g[b] = dir ? R(2.0 * w15(b)) * (tw - T_ref) - gv : gv;
+                    const R gv = load_link<S, kRaw>(gin, og, R(w15(b)) * T_ref);
+                    g[b] = dir ? anti_bounce<S, kRaw>(gv, w15(b), tw, T_ref) : gv;
                 }
             }
         }
@@ -181,7 +176,7 @@ __global__ void __launch_bounds__(kTmaTX * TY + 32, TmaLayout<typename S::T, TY>
     step_d3q27_tma_kernel(const __grid_constant__ CUtensorMap mf, const __grid_constant__ CUtensorMap mg,
                           const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                           typename S::T* __restrict__ fout, typename S::T* __restrict__ gout,
-                          Geometry geo, Coeffs3D<typename S::R> c, unsigned* status, int tiles_x,
+                          Geometry geo, StepCoeffs3D<S, kRates> c, unsigned* status, int tiles_x,
                           int tiles_y, int n_tiles)
 {
     using R = typename S::R;
@@ -265,21 +260,22 @@ __global__ void __launch_bounds__(kTmaTX * TY + 32, TmaLayout<typename S::T, TY>
                     const T* sb = reinterpret_cast<const T*>(smem + st * L::kStageBytes) + ly * L::kBoxX + lx + L::kHalo;
                     static_for<27>([&](auto A) {
                         constexpr int a = decltype(A)::value;
-                        f[a] = dev_of<S>(sb[a * L::kSlabElems - e27(a, 0)], R(w27(a)));
+                        f[a] = staged_value<S, kRates == 3>(sb[a * L::kSlabElems - e27(a, 0)]);
                     });
                     static_for<15>([&](auto B) {
                         constexpr int b = decltype(B)::value;
-                        g[b] = dev_of<S>(sb[(27 + b) * L::kSlabElems - e15(b, 0)], R(w15(b)) * c.T_ref);
+                        g[b] = staged_value<S, kRates == 3>(sb[(27 + b) * L::kSlabElems - e15(b, 0)]);
                     });
                     if (x == 0 || x == geo.nx - 1)
-                        fix_x_edge_d3q27<S, Idx>(fin, gin, geo, x, y, z, i, c.T_ref, f, g);
+                        fix_x_edge_d3q27<S, Idx, kRates == 3>(fin, gin, geo, x, y, z, i, c.T_ref, f, g);
                 } else if (x > 0 && x < geo.nx - 1 && y > 0 && y < geo.ny - 1 && z > 0 && z < geo.nz - 1) {
-                    pull_d3q27_d3q15_interior<S, Idx>(fin, gin, geo, i, c.T_ref, f, g);
+                    pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
                 } else {
                     const NodeWalls<R> w = node_walls<R>(geo, x, y, z, 3);
-                    pull_d3q27_d3q15<S, Idx>(fin, gin, geo, w, i, c.T_ref, f, g);
+                    pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
                 }
-                collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);
+                if constexpr (kRates == 3) collide_store_d3q27_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
+                else collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(empty_bar(st));   // this warp is done with stage st

@@ -22,7 +22,9 @@ if not torch.cuda.is_available():
 from paper_2504_09041_gb300 import lbm as L  # noqa: E402
 
 BOXES = [(2, "cavity", (1, 33, 70)), (2, "rb", (1, 19, 131)), (2, "periodic", (1, 64, 32)),
-         (2, "cavity", (1, 3, 2)), (2, "rb", (1, 1, 5))]
+         (2, "cavity", (1, 3, 2)), (2, "rb", (1, 1, 5)),
+         (3, "cavity", (13, 21, 37)), (3, "mixed3d", (9, 10, 70)), (3, "periodic", (5, 6, 33)),
+         (3, "mixed3d", (2, 3, 1))]
 
 
 @pytest.mark.parametrize("gbeta", [None, 3e-3])
