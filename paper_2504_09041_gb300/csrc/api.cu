@@ -286,7 +286,7 @@ int plan_box(int lattice, int nx, int ny, int nz, double Ra, double Pr, double M
     hc.gaxis = bc->gravity_axis;
     hc.fp16_sr = 1;
     hc.adj_sync = 2;   // adjoint step: 128 x 2 blocks with phase barriers (measured fastest)
-    hc.rows3d = 0;     // 3D FP32 / FP16S step: rows per thread chosen per form (rows3d_for)
+    hc.rows3d = 0;     // 3D FP32 / FP16S step: rows per thread chosen by rows3d_for
     const double om_nu = 1.0 / (3.0 * P->nu + 0.5);
     const double om_alpha = 1.0 / (3.0 * P->alpha + 0.5);
     // App. A, B, C: shear / diffusivity rates from nu / alpha, bulk and every free rate 1
@@ -543,7 +543,7 @@ int lbm_info(lbm_handle h, lbm_info_t* o)
     o->steps = h->steps;
     o->bytes_per_node_update = 2.0 * (h->qf + h->qg) * (double)lbm::storage_bytes(h->prec);
     o->state_bytes = kStateHeader + pop_bytes(h);
-    const dim3 b = lbm::block_shape(h->nx, dim3(h->block_x, h->block_y, 1), h->dim);
+    const dim3 b = lbm::block_shape(h->geo, h->prec, h->dim, dim3(h->block_x, h->block_y, 1));
     o->block_x = (int)b.x;
     o->block_y = (int)b.y;
     o->graph_steps = h->graph_steps;

@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(256, BatchBounds<S>::kMinBlocks)
         if (__ldg(&members[mid].tile0) <= t0) lo = mid;
         else hi = mid - 1;
     }
+    wait_previous_step();
     int k = lo, held = -1;
     for (int t = t0; t < t1; ++t) {
         while (k + 1 < n_members && __ldg(&members[k + 1].tile0) <= t) ++k;
@@ -116,10 +117,9 @@ static cudaError_t launch_batch(const void* fin, const void* gin, void* fout, vo
                                 int tile_y, int grid, unsigned* status, cudaStream_t st)
 {
     using T = typename S::T;
-    batch_step_d2q9_kernel<S><<<grid, tile_x * tile_y, 0, st>>>(
-        (const T*)fin, (const T*)gin, (T*)fout, (T*)gout,
-        (const BatchMember<S>*)members, n_members, n_tiles, tile_x, tile_y, status);
-    return cudaGetLastError();
+    return launch_step_kernel(batch_step_d2q9_kernel<S>, dim3(grid), dim3(tile_x * tile_y), st, (const T*)fin,
+                              (const T*)gin, (T*)fout, (T*)gout, (const BatchMember<S>*)members, n_members,
+                              n_tiles, tile_x, tile_y, status);
 }
 
 }  // namespace lbm

@@ -128,6 +128,23 @@ cudaError_t launch_adjoint_step_d2q9(int prec, int arith, const void* f_prev, co
 
 namespace lbm {
 
+// Launch of a kernel that calls wait_previous_step: its blocks may start while the kernel before it on
+// the stream is still running (a predecessor that is no kernel is waited for as usual).
+template <class... P, class... A>
+inline cudaError_t launch_step_kernel(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <class R, int QF, int QG>
 inline Coeffs<R, QF, QG> make_coeffs(const HostCoeffs& h)
 {
@@ -170,15 +187,25 @@ inline auto make_step_coeffs(const HostCoeffs& h)
 }
 
 // Default thread blocks, x-major so that a warp reads and writes 32 consecutive nodes; a
-// caller-chosen shape (block.x > 0) replaces it.  2D: 256 threads.  3D: 64 x 1, which at 96
-// registers per thread lets 10 blocks (20 warps) share an SM against 16 warps for 256-thread
-// blocks (measured on the 256^3 cavity: 16.4 vs 15.8 GLUPS).
-inline dim3 block_shape(int nx, dim3 chosen = dim3(0, 0, 0), int dim = 2)
+// caller-chosen shape (block.x > 0) replaces it.
+// 2D, FP64: one warp, so that few warps spread over all SMs: an SM takes one FP64 warp instruction per 19
+//   cycles and a sub-partition one per 64, so 64^2 nodes (128 warps) take 8.1 us a step on 128 SMs
+//   against 15.8 in blocks of 256 threads on 16; 1024 x 512 takes 189.7 us against 196 (a finer tail).
+//   Above 65535 rows two warps, the launch grid's limit.
+// 2D, FP32 and FP16 storage: 64 x 2 (1024 x 512 FP32 9.97 us against 10.13 for 256 threads, 512^2 5.77
+//   against 5.95, 64^2 1.80 against 2.15; one warp per block runs at 16.9, bound by block turnover).
+// 3D: 64 x 1, which at 72-96 registers per thread lets 10-14 blocks share an SM against four of 256
+//   threads (256^3 FP32: 16.4 against 15.8 GLUPS); 32 x 1 where a row ends in a half-empty block
+//   (131 x 93 x 77: FP32 64.0 us against 68.7, FP16S 45.3 against 51.7, FP64 1273 against 1288);
+//   128 x 1 from two million nodes on, where rows fill such blocks (256^3: FP32 849 us against 853,
+//   FP16S 826 against 832; but 64^3 15.8 against 14.5).
+inline dim3 block_shape(const Geometry& g, int prec, int dim, dim3 chosen = dim3(0, 0, 0))
 {
     if (chosen.x > 0) return dim3(chosen.x, chosen.y, 1);
-    if (dim == 3) return dim3(nx > 32 ? 64 : 32, 1, 1);
-    const int bx = nx >= 128 ? 128 : ((nx + 31) / 32) * 32;
-    return dim3(bx, 256 / bx, 1);
+    const int warps = (g.nx + 31) / 32;   // per row
+    if (dim == 3) return dim3(warps & 1 ? 32 : (warps & 3 || g.n < (1 << 21) ? 64 : 128), 1, 1);
+    if (prec == kF64) return dim3(32, g.ny > 65535 ? 2 : 1, 1);
+    return g.nx > 32 ? dim3(64, 2, 1) : dim3(32, 4, 1);
 }
 
 // 32-bit element offsets suffice when every population plane index q * n fits in 32 bits.
@@ -233,15 +260,10 @@ inline int rate_class(const HostCoeffs& h)
     return h.gaxis == 2 ? 3 : 2;
 }
 
-// Rows per thread of the 3D FP32 / FP16S step: the handle's setting, or when that is 0 the faster
-// one measured on the 256^3 cavity: one for FP16S storage with the reduced collisions of the
-// default rates (+0.8 % against two), two otherwise (FP32 +1.2 % at its 72 registers; FP16S with
-// the general collision +0.5-0.9 %).
-inline int rows3d_for(const HostCoeffs& h, bool f16s)
-{
-    if (h.rows3d > 0) return h.rows3d;
-    return f16s && rate_class(h) >= 2 ? 1 : 2;
-}
+// Rows per thread of the 3D FP32 / FP16S step: the handle's setting, or when that is 0 one, the
+// fastest with every collision (FP32 128^3 106 us against 111 for two rows, 256^3 853 against 862,
+// 32^3 4.1 against 5.7; only the general collision at 256^3 is within 0.2 % either way).
+inline int rows3d_for(const HostCoeffs& h) { return h.rows3d > 0 ? h.rows3d : 1; }
 
 inline dim3 grid_shape(const Geometry& g, dim3 b)
 {

@@ -16,6 +16,56 @@ namespace lbm {
 
 enum FaceKind { kPeriodic = 0, kAdiabatic = 1, kFixedT = 2 };
 
+// 2D steps of one time loop are launched as programmatic dependents (launch_step_kernel): a step's
+// blocks may start while the previous step drains, wait here for it to complete before their first
+// access to populations, and only then let the step after them start, so at most two steps are ever
+// in flight.  That hides the launch (a step of 64^2 nodes: FP64 8.58 -> 8.07 us, FP32 1.86 -> 1.80; 256^2
+// FP32 2.64 -> 2.56).  The 3D steps are launched one after the other: their times do not change, and
+// in FP64 blocks that wait beside running ones share the sub-partitions' FP64 units unevenly (32^3: 67
+// us against 41).
+__device__ __forceinline__ void wait_previous_step()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Loads of populations: ld_ro through the read-only path, ld_step in kernels that call
+// wait_previous_step, whose predecessor writes what they read (volatile, so that they stay behind the
+// wait, and not the read-only path).  FP32 and FP16 carry an L2 prefetch hint of 256 bytes: the pull
+// reads every population plane in full, so the sectors around each warp's row are always used by
+// the neighbouring warps.
+__device__ __forceinline__ double ld_ro(const double* p) { return __ldg(p); }
+__device__ __forceinline__ float ld_ro(const float* p)
+{
+    float v;
+    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_ro(const __half* p)
+{
+    unsigned short v;
+    asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+__device__ __forceinline__ double ld_step(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_step(const float* p)
+{
+    float v;
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_step(const __half* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+
 // Storage policies: the type in HBM and the type of the moment algebra in registers.  The
 // kernels work on deviations from the rest populations (f_a - w_a and g_a - w_a T_o), which keeps
 // every quantity of the collision small and resolves it to the register type's precision.
@@ -25,7 +75,7 @@ enum FaceKind { kPeriodic = 0, kAdiabatic = 1, kFixedT = 2 };
 //    normal range (full 11-bit significand) while |deviation| < 64 still fits; the scale is a
 //    power of two and adds no rounding.
 //
-// The reduced steps (default rates and gravity axis; FP64 and F16S) take the stored number itself (load_raw) and
+// The reduced steps (default rates and gravity axis; FP64 and F16S) take the stored number itself (raw) and
 // work in its units: every relation of the step is homogeneous of degree one in the populations, so
 // multiplying them all by kUnits only multiplies the rest state's constants.  kFull: the stored
 // number is the population, not its deviation; the rest state is then taken off in the raw sums.
@@ -34,30 +84,14 @@ struct StoreF64 {
     using R = double;
     static constexpr bool kFull = true;
     static constexpr double kUnits = 1.0;
-    __device__ static R load_raw(const T* p, size_t i) { return __ldg(p + i); }
-    __device__ static R load_dev(const T* p, size_t i, R shift) { return __ldg(p + i) - shift; }
+    __device__ static R raw(T v) { return v; }
+    __device__ static R dev(T v, R shift) { return v - shift; }
     __device__ static void store_dev(T* p, size_t i, R dev, R shift) { p[i] = shift + dev; }
 };
-// Read-only loads with an L2 prefetch hint of 256 bytes: the pull reads every population plane in
-// full, so the sectors around each warp's row are always used by the neighbouring warps.
-__device__ __forceinline__ float ldg_pf256(const float* p)
-{
-    float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
-__device__ __forceinline__ __half ldg_pf256(const __half* p)
-{
-    unsigned short v;
-    asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
-    return __ushort_as_half(v);
-}
-
 struct StoreF32 {
     using T = float;
     using R = float;
-    __device__ static R load_dev(const T* p, size_t i, R) { return ldg_pf256(p + i); }
+    __device__ static R dev(T v, R) { return v; }
     __device__ static void store_dev(T* p, size_t i, R dev, R) { p[i] = dev; }
 };
 struct StoreF16S {
@@ -68,11 +102,8 @@ struct StoreF16S {
     static constexpr float kInvScale = 1.0f / 1024.0f;
     static constexpr bool kFull = false;
     static constexpr double kUnits = 1024.0;
-    __device__ static R load_raw(const T* p, size_t i) { return __half2float(ldg_pf256(p + i)); }
-    __device__ static R load_dev(const T* p, size_t i, R)
-    {
-        return __half2float(ldg_pf256(p + i)) * kInvScale;
-    }
+    __device__ static R raw(T v) { return __half2float(v); }
+    __device__ static R dev(T v, R) { return __half2float(v) * kInvScale; }
     __device__ static void store_dev(T* p, size_t i, R dev, R) { p[i] = __float2half_rn(dev * kScale); }
     // a deviation already multiplied by kScale
     __device__ static void store_scaled(T* p, size_t i, R scaled) { p[i] = __float2half_rn(scaled); }
@@ -281,21 +312,30 @@ __device__ __forceinline__ int link_source(const Geometry& g, const NodeWalls<R>
     return s;
 }
 
-// Stored numbers at one link, for a population (load_dev) or in storage units (load_raw).
-template <class S, bool kRaw, class Idx>
+// How a pull reads populations.
+enum Pull {
+    kPullDev = 0,    // deviations
+    kPullRaw = 1,    // stored numbers, for the reduced steps
+    kPullAfter = 2   // flag: in a kernel that has called wait_previous_step
+};
+
+template <class S, int kPull, class Idx>
 __device__ __forceinline__ typename S::R load_link(const typename S::T* p, Idx off, typename S::R shift)
 {
-    if constexpr (kRaw) return S::load_raw(p, off);
-    else return S::load_dev(p, off, shift);
+    typename S::T v;
+    if constexpr ((kPull & kPullAfter) != 0) v = ld_step(p + off);
+    else v = ld_ro(p + off);
+    if constexpr ((kPull & kPullRaw) != 0) return S::raw(v);
+    else return S::dev(v, shift);
 }
 // Anti-bounce-back of the energy population gv against a wall at temperature tw (link weight w), in
 // the units of load_link.
-template <class S, bool kRaw>
+template <class S, int kPull>
 __device__ __forceinline__ typename S::R anti_bounce(typename S::R gv, double w, typename S::R tw,
                                                      typename S::R T_ref)
 {
     using R = typename S::R;
-    if constexpr (kRaw) {
+    if constexpr ((kPull & kPullRaw) != 0) {
         if constexpr (S::kFull) return R(2.0 * w) * tw - gv;
         else return R(2.0 * S::kUnits * w) * (tw - T_ref) - gv;
     } else {

@@ -81,7 +81,7 @@ __device__ __forceinline__ double pulled_T(const typename S::T* g, const Geometr
             R tw;
             const int s = link_source<e9(a, 0), e9(a, 1), 0>(geo, w, i, &out, &dir, &tw);
             const size_t off = out ? (size_t)opp9(a) * geo.n + i : (size_t)a * geo.n + s;
-            const R gv = S::load_dev(g, off, R(w9(a)) * R(T_ref));
+            const R gv = S::dev(ld_ro(g + off), R(w9(a)) * R(T_ref));
             sum += (double)(dir ? R(2.0 * w9(a)) * (tw - R(T_ref)) - gv : gv);
         });
     } else {
@@ -91,7 +91,7 @@ __device__ __forceinline__ double pulled_T(const typename S::T* g, const Geometr
             R tw;
             const int s = link_source<e15(b, 0), e15(b, 1), e15(b, 2)>(geo, w, i, &out, &dir, &tw);
             const size_t off = out ? (size_t)opp15(b) * geo.n + i : (size_t)b * geo.n + s;
-            const R gv = S::load_dev(g, off, R(w15(b)) * R(T_ref));
+            const R gv = S::dev(ld_ro(g + off), R(w15(b)) * R(T_ref));
             sum += (double)(dir ? R(2.0 * w15(b)) * (tw - R(T_ref)) - gv : gv);
         });
     }

@@ -10,18 +10,14 @@ static cudaError_t run_as(const void* fin, const void* gin, void* fout, void* go
 {
     using T = typename S::T;
     using R = typename S::R;
-    const dim3 b = block_shape(geo.nx, block);
+    const int prec = std::is_same<S, StoreF64>::value ? kF64 : (std::is_same<S, StoreF32>::value ? kF32 : kF16S);
+    const dim3 b = block_shape(geo, prec, 2, block);
     const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
     StepCoeffs2D<S, kUnit> c;
     if constexpr (kUnit) c = make_unit_coeffs<R, 2>(hc);
     else c = make_coeffs<R, 9, 9>(hc);
-    if (step_index32(geo, 9, hc))
-        step_d2q9_kernel<S, unsigned, kUnit><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
-                                                                 (T*)gout, geo, c, status);
-    else
-        step_d2q9_kernel<S, size_t, kUnit><<<grid, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout,
-                                                               (T*)gout, geo, c, status);
-    return cudaGetLastError();
+    auto kern = step_index32(geo, 9, hc) ? step_d2q9_kernel<S, unsigned, kUnit> : step_d2q9_kernel<S, size_t, kUnit>;
+    return launch_step_kernel(kern, grid, b, st, (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
 }
 
 template <class S>

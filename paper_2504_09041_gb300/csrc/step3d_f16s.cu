@@ -16,25 +16,17 @@ static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fou
     using S = StoreF16S;
     using T = typename S::T;
     using R = typename S::R;
-    const dim3 b = block_shape(geo.nx, block, 3);
+    const dim3 b = block_shape(geo, kF16S, 3, block);
     const auto c = make_step_coeffs<R, kU>(hc);
-    const int rows = rows3d_for(hc, true);
-    if (step_index32(geo, 27, hc) && rows == 2) {
-        dim3 g = grid_shape(geo, b);
-        g.y = (g.y + 1) / 2;
-        step_d3q27_kernel<S, unsigned, 2, kU><<<g, b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
-    } else if (step_index32(geo, 27, hc) && rows == 4) {
-        dim3 g = grid_shape(geo, b);
-        g.y = (g.y + 3) / 4;
-        step_d3q27_kernel<S, unsigned, 4, kU><<<g, b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
-    } else if (step_index32(geo, 27, hc))
-        step_d3q27_kernel<S, unsigned, 1, kU><<<grid_shape(geo, b), b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
-    else
-        step_d3q27_kernel<S, size_t, 1, kU><<<grid_shape(geo, b), b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    const bool idx32 = step_index32(geo, 27, hc);
+    const int rows = idx32 ? rows3d_for(hc) : 1;
+    auto kern = !idx32 ? step_d3q27_kernel<S, size_t, 1, kU>
+                : rows == 4 ? step_d3q27_kernel<S, unsigned, 4, kU>
+                : rows == 2 ? step_d3q27_kernel<S, unsigned, 2, kU>
+                            : step_d3q27_kernel<S, unsigned, 1, kU>;
+    dim3 g = grid_shape(geo, b);
+    g.y = (g.y + rows - 1) / rows;
+    kern<<<g, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
     return cudaGetLastError();
 }
 

@@ -14,14 +14,10 @@ static cudaError_t launch_plain_f64(const void* fin, const void* gin, void* fout
     using S = StoreF64;
     using T = typename S::T;
     using R = typename S::R;
-    const dim3 b = block_shape(geo.nx, block, 3);
+    const dim3 b = block_shape(geo, kF64, 3, block);
     const auto c = make_step_coeffs<R, kU>(hc);
-    if (step_index32(geo, 27, hc))
-        step_d3q27_kernel<S, unsigned, 1, kU><<<grid_shape(geo, b), b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
-    else
-        step_d3q27_kernel<S, size_t, 1, kU><<<grid_shape(geo, b), b, 0, st>>>(
-            (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    auto kern = step_index32(geo, 27, hc) ? step_d3q27_kernel<S, unsigned, 1, kU> : step_d3q27_kernel<S, size_t, 1, kU>;
+    kern<<<grid_shape(geo, b), b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
     return cudaGetLastError();
 }
 

@@ -24,7 +24,7 @@ using Coeffs2D = Coeffs<R, 9, 9>;
 // bounce-back (adiabatic) or anti-bounce-back (fixed T) for g at the walls (Sec. 6.1), in
 // deviations: the anti-bounce-back g_a = -g~_abar + 2 w_a T_w becomes
 // gamma_a = -gamma~_abar + 2 w_a (T_w - T_o).
-template <class S, class Idx = size_t, bool kRaw = false>
+template <class S, class Idx = size_t, int kPull = kPullDev>
 __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
                                           const typename S::T* __restrict__ gin, const Geometry& geo,
                                           const NodeWalls<typename S::R>& w, int i, typename S::R T_ref,
@@ -38,15 +38,15 @@ __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
         R tw;
         const int s = link_source<e9(a, 0), e9(a, 1), 0>(geo, w, i, &out, &dir, &tw);
         const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-        f[a] = load_link<S, kRaw>(fin, off, R(w9(a)));
-        const R gv = load_link<S, kRaw>(gin, off, R(w9(a)) * T_ref);
-        g[a] = dir ? anti_bounce<S, kRaw>(gv, w9(a), tw, T_ref) : gv;
+        f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
+        const R gv = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
+        g[a] = dir ? anti_bounce<S, kPull>(gv, w9(a), tw, T_ref) : gv;
     });
 }
 
 // The same pull at a node whose eight neighbours all lie inside the box: no wall and no
 // periodic wrap touches any link, so every population comes straight from its upwind node.
-template <class S, class Idx = size_t, bool kRaw = false>
+template <class S, class Idx = size_t, int kPull = kPullDev>
 __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restrict__ fin,
                                                    const typename S::T* __restrict__ gin,
                                                    const Geometry& geo, int i, typename S::R T_ref,
@@ -56,8 +56,8 @@ __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restri
     static_for<9>([&](auto A) {
         constexpr int a = decltype(A)::value;
         const Idx off = (Idx)a * geo.n + (i - (e9(a, 0) + e9(a, 1) * geo.nx));
-        f[a] = load_link<S, kRaw>(fin, off, R(w9(a)));
-        g[a] = load_link<S, kRaw>(gin, off, R(w9(a)) * T_ref);
+        f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
+        g[a] = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
     });
 }
 
@@ -172,7 +172,7 @@ __device__ __forceinline__ void from_central_d2q9(R p[3][3], R f[9], R ux, R uy)
 }
 
 // Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
-// y (unit_rates_2d, checked by the host), from the stored numbers in f and g (load_raw).  Used for FP64
+// y (unit_rates_2d, checked by the host), from the stored numbers in f and g (raw).  Used for FP64
 // storage, bound by the FP64 pipe, and FP16 storage, bound by issue; FP32 storage, bound by the
 // memory, keeps the general collision and with it its rounding.
 //
@@ -378,6 +378,7 @@ __device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__
                                                int x, int y)
 {
     using R = typename S::R;
+    constexpr int kPull = kPullAfter | (kUnit ? kPullRaw : kPullDev);
     const int i = x + geo.nx * y;
     R f[9], g[9];
     // Which pull: decided per warp where possible, so that a warp holding an x-wall node of an
@@ -386,15 +387,15 @@ __device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__
     const bool in = y_in && x > 0 && x < geo.nx - 1;
     const unsigned lanes = __activemask();
     if (__all_sync(lanes, in)) {
-        pull_d2q9_interior<S, Idx, kUnit>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d2q9_interior<S, Idx, kPull>(fin, gin, geo, i, c.T_ref, f, g);
     } else if (__all_sync(lanes, y_in)) {
         const NodeWalls<R> w = node_walls_x<R>(geo, x, y, 0);
-        pull_d2q9<S, Idx, kUnit>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d2q9<S, Idx, kPull>(fin, gin, geo, w, i, c.T_ref, f, g);
     } else if (in) {
-        pull_d2q9_interior<S, Idx, kUnit>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d2q9_interior<S, Idx, kPull>(fin, gin, geo, i, c.T_ref, f, g);
     } else {
         const NodeWalls<R> w = node_walls<R>(geo, x, y, 0, 2);
-        pull_d2q9<S, Idx, kUnit>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d2q9<S, Idx, kPull>(fin, gin, geo, w, i, c.T_ref, f, g);
     }
 
     if constexpr (kUnit) {
@@ -411,6 +412,7 @@ __global__ void __launch_bounds__(256)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    wait_previous_step();
     if (x >= geo.nx || y >= geo.ny) return;
     node_step_d2q9<S, Idx, kUnit>(fin, gin, fout, gout, geo, c, status, x, y);
 }

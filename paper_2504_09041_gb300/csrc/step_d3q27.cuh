@@ -33,7 +33,7 @@ __host__ __device__ constexpr int g15_of_27(int a)
     return a < 7 ? a : (a >= 19 ? a - 12 : -1);
 }
 
-template <class S, class Idx = size_t, bool kRaw = false>
+template <class S, class Idx = size_t, int kPull = kPullDev>
 __device__ __forceinline__ void pull_d3q27_d3q15(const typename S::T* __restrict__ fin,
                                                  const typename S::T* __restrict__ gin,
                                                  const Geometry& geo,
@@ -49,19 +49,19 @@ __device__ __forceinline__ void pull_d3q27_d3q15(const typename S::T* __restrict
         R tw;
         const int s = link_source<e27(a, 0), e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
         const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-        f[a] = load_link<S, kRaw>(fin, off, R(w27(a)));
+        f[a] = load_link<S, kPull>(fin, off, R(w27(a)));
         constexpr int b = g15_of_27(a);
         if constexpr (b >= 0) {
             constexpr int ob = opp15(b);
             const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
-            const R gv = load_link<S, kRaw>(gin, og, R(w15(b)) * T_ref);
-            g[b] = dir ? anti_bounce<S, kRaw>(gv, w15(b), tw, T_ref) : gv;
+            const R gv = load_link<S, kPull>(gin, og, R(w15(b)) * T_ref);
+            g[b] = dir ? anti_bounce<S, kPull>(gv, w15(b), tw, T_ref) : gv;
         }
     });
 }
 
 // The same pull at a node whose 26 neighbours all lie inside the box (no wall, no wrap).
-template <class S, class Idx = size_t, bool kRaw = false>
+template <class S, class Idx = size_t, int kPull = kPullDev>
 __device__ __forceinline__ void pull_d3q27_d3q15_interior(const typename S::T* __restrict__ fin,
                                                           const typename S::T* __restrict__ gin,
                                                           const Geometry& geo, int i,
@@ -72,9 +72,9 @@ __device__ __forceinline__ void pull_d3q27_d3q15_interior(const typename S::T* _
     static_for<27>([&](auto A) {
         constexpr int a = decltype(A)::value;
         const int s = i - (e27(a, 0) + e27(a, 1) * geo.nx + e27(a, 2) * geo.nxy);
-        f[a] = load_link<S, kRaw>(fin, (Idx)((Idx)a * geo.n + s), R(w27(a)));
+        f[a] = load_link<S, kPull>(fin, (Idx)((Idx)a * geo.n + s), R(w27(a)));
         constexpr int b = g15_of_27(a);
-        if constexpr (b >= 0) g[b] = load_link<S, kRaw>(gin, (Idx)((Idx)b * geo.n + s), R(w15(b)) * T_ref);
+        if constexpr (b >= 0) g[b] = load_link<S, kPull>(gin, (Idx)((Idx)b * geo.n + s), R(w15(b)) * T_ref);
     });
 }
 
@@ -573,7 +573,7 @@ __device__ __forceinline__ void raw01_g_d3q15(const R g[15], R& r000, R& r100, R
 }
 
 // Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
-// z (rate_class 3, checked by the host), from the stored numbers in f and g (load_raw); the 3D
+// z (rate_class 3, checked by the host), from the stored numbers in f and g (raw); the 3D
 // counterpart of collide_store_d2q9_unit, see there.  Of the flow's moments only those enter that
 // relax with a rate of their own (rho, j and order 2) or that the force multiplies (orders 0-1 in z, up
 // to 2 in x and y); t_210 and t_120 vanish.  The relaxed moments are held as deviations e from the
@@ -834,15 +834,15 @@ __device__ __forceinline__ void node_step_d3q27(const typename S::T* __restrict_
     const bool in = yz_in && x > 0 && x < geo.nx - 1;
     const unsigned lanes = __activemask();
     if (__all_sync(lanes, in)) {
-        pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d3q27_d3q15_interior<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, i, c.T_ref, f, g);
     } else if (__all_sync(lanes, yz_in)) {
         const NodeWalls<R> w = node_walls_x<R>(geo, x, y, z);
-        pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d3q27_d3q15<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, w, i, c.T_ref, f, g);
     } else if (in) {
-        pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
+        pull_d3q27_d3q15_interior<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, i, c.T_ref, f, g);
     } else {
         const NodeWalls<R> w = node_walls<R>(geo, x, y, z, 3);
-        pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
+        pull_d3q27_d3q15<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, w, i, c.T_ref, f, g);
     }
     if constexpr (kRates == 3) collide_store_d3q27_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
     else collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);

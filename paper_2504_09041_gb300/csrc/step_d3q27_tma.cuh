@@ -107,11 +107,11 @@ __device__ __forceinline__ void fence_mbar_init()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// Value of a stored element: its deviation from the rest state, or with kRaw in storage units.
-template <class S, bool kRaw>
+// Value of a stored element: its deviation from the rest state, or in storage units (kPullRaw).
+template <class S, int kPull>
 __device__ __forceinline__ typename S::R staged_value(typename S::T v)
 {
-    if constexpr (std::is_same<S, StoreF16S>::value) return __half2float(v) * (kRaw ? 1.0f : S::kInvScale);
+    if constexpr (std::is_same<S, StoreF16S>::value) return __half2float(v) * ((kPull & kPullRaw) != 0 ? 1.0f : S::kInvScale);
     else return v;
 }
 
@@ -133,7 +133,7 @@ __device__ __forceinline__ void tma_issue_tile(const CUtensorMap* mf, const CUte
 
 // Links of a node on an x wall (or x wrap) that leave the box through x, replaced by the wall
 // rules (or the wrapped source) from global memory; the other links keep their staged values.
-template <class S, class Idx, bool kRaw>
+template <class S, class Idx, int kPull>
 __device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict__ fin,
                                                  const typename S::T* __restrict__ gin,
                                                  const Geometry& geo, int x, int y, int z, int i,
@@ -153,13 +153,13 @@ __device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict
                 R tw;
                 const int s = link_source<ex, e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
                 const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-                f[a] = load_link<S, kRaw>(fin, off, R(w27(a)));
+                f[a] = load_link<S, kPull>(fin, off, R(w27(a)));
                 constexpr int b = g15_of_27(a);
                 if constexpr (b >= 0) {
                     constexpr int ob = opp15(b);
                     const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
-                    const R gv = load_link<S, kRaw>(gin, og, R(w15(b)) * T_ref);
-                    g[b] = dir ? anti_bounce<S, kRaw>(gv, w15(b), tw, T_ref) : gv;
+                    const R gv = load_link<S, kPull>(gin, og, R(w15(b)) * T_ref);
+                    g[b] = dir ? anti_bounce<S, kPull>(gv, w15(b), tw, T_ref) : gv;
                 }
             }
         }
@@ -260,19 +260,19 @@ __global__ void __launch_bounds__(kTmaTX * TY + 32, TmaLayout<typename S::T, TY>
                     const T* sb = reinterpret_cast<const T*>(smem + st * L::kStageBytes) + ly * L::kBoxX + lx + L::kHalo;
                     static_for<27>([&](auto A) {
                         constexpr int a = decltype(A)::value;
-                        f[a] = staged_value<S, kRates == 3>(sb[a * L::kSlabElems - e27(a, 0)]);
+                        f[a] = staged_value<S, kRates == 3 ? kPullRaw : kPullDev>(sb[a * L::kSlabElems - e27(a, 0)]);
                     });
                     static_for<15>([&](auto B) {
                         constexpr int b = decltype(B)::value;
-                        g[b] = staged_value<S, kRates == 3>(sb[(27 + b) * L::kSlabElems - e15(b, 0)]);
+                        g[b] = staged_value<S, kRates == 3 ? kPullRaw : kPullDev>(sb[(27 + b) * L::kSlabElems - e15(b, 0)]);
                     });
                     if (x == 0 || x == geo.nx - 1)
-                        fix_x_edge_d3q27<S, Idx, kRates == 3>(fin, gin, geo, x, y, z, i, c.T_ref, f, g);
+                        fix_x_edge_d3q27<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, x, y, z, i, c.T_ref, f, g);
                 } else if (x > 0 && x < geo.nx - 1 && y > 0 && y < geo.ny - 1 && z > 0 && z < geo.nz - 1) {
-                    pull_d3q27_d3q15_interior<S, Idx, kRates == 3>(fin, gin, geo, i, c.T_ref, f, g);
+                    pull_d3q27_d3q15_interior<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, i, c.T_ref, f, g);
                 } else {
                     const NodeWalls<R> w = node_walls<R>(geo, x, y, z, 3);
-                    pull_d3q27_d3q15<S, Idx, kRates == 3>(fin, gin, geo, w, i, c.T_ref, f, g);
+                    pull_d3q27_d3q15<S, Idx, kRates == 3 ? kPullRaw : kPullDev>(fin, gin, geo, w, i, c.T_ref, f, g);
                 }
                 if constexpr (kRates == 3) collide_store_d3q27_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
                 else collide_store_d3q27<S, Idx, kRates>(f, g, fout, gout, geo, c, status, i);
