@@ -170,10 +170,6 @@ inline UnitCoeffs<R> make_unit_coeffs(const HostCoeffs& h)
     for (int b = 1; b < 4; ++b) c.kg[b - 1] = R(1.0 - h.om_g[b]);
     c.gbeta = R(h.gbeta);
     c.T_ref = R(h.T_ref);
-    c.T_ref6 = R(h.T_ref / 6.0);
-    c.T_ref23 = R(h.T_ref * (2.0 / 3.0));
-    const double w[3] = {DIM == 2 ? w9(0) : w15(0), DIM == 2 ? w9(1) : w15(1), DIM == 2 ? w9(8) : w15(14)};
-    for (int k = 0; k < 3; ++k) c.wT[k] = R(w[k]) * R(h.T_ref);
     c.fp16_sr = h.fp16_sr;
     return c;
 }

@@ -188,8 +188,6 @@ struct UnitCoeffs {
     R kf[6];             // 1 - omega of flow slots 4 .. 9
     R kg[3];             // 1 - omega of energy slots 1 .. 3
     R gbeta, T_ref;
-    R T_ref6, T_ref23;   // T_ref / 6 and 2 T_ref / 3: the rest state's share of an outer and a middle line
-    R wT[3];             // rest weights of the energy (centre, axis, corner links) times T_ref
     int fp16_sr;         // as in Coeffs
 };
 

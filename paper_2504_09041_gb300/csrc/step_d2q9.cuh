@@ -215,18 +215,17 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
     const R Myy = k0[0] + k0[2], drho = Myy + k0[1];
     const R jx = (d[0] + d[2]) + d[1], jy = k0[2] - k0[0];
     const R Mxx = (s[0] + s[2]) + s[1], Mxy = d[2] - d[0], Mxxy = s[2] - s[0];
-    // raw sums of the energy
-    const R T0 = S::kFull ? c.T_ref : R(kS) * c.T_ref;
-    const R top = g[2] + (g[5] + g[6]), bot = g[4] + (g[7] + g[8]);
-    const R g0 = S::kFull ? g[0] - T0 : g[0];
-    const R dT = (g0 + (g[1] + g[3])) + (top + bot);
-    const R jgy = top - bot;
-    const R jgx = (g[1] - g[3]) + ((g[5] - g[6]) + (g[8] - g[7]));
-    const R T = T0 + dT, rho = R(kS) + drho;
+    // raw sums of the energy, over opposite links: g = dT + T0.  Stored populations are summed as they
+    // are (T0 = 0), which also keeps the small ones beside a cold wall exact.
+    const R T0 = S::kFull ? R(0) : R(kS) * c.T_ref;
+    const R dT = (g[0] + ((g[1] + g[3]) + (g[2] + g[4]))) + ((g[5] + g[7]) + (g[6] + g[8]));
+    const R d57 = g[5] - g[7], d68 = g[6] - g[8];
+    const R jgx = (g[1] - g[3]) + (d57 - d68), jgy = (g[2] - g[4]) + (d57 + d68);
+    const R T = S::kFull ? dT : T0 + dT, rho = R(kS) + drho;
     check_node_bits(status, rho, T);
 
     const R irho = recip(rho);
-    const R Fy = c.gbeta * dT, hF = half * Fy;
+    const R Fy = c.gbeta * (S::kFull ? dT - c.T_ref : dT), hF = half * Fy;
     const R py = jy + hF;                        // rho u_y
     const R ux = jx * irho, uy = py * irho;
     const R uxh = half * ux, uyh = half * uy;
@@ -274,7 +273,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
     {
         const R t10 = c.kg[0] * (jgx - ux * T);
         const R t01 = c.kg[1] * (jgy - uy * T);
-        const R T6 = R(1.0 / 6.0) * T, dT6 = R(1.0 / 6.0) * dT;
+        const R dT6 = R(1.0 / 6.0) * dT, T6 = S::kFull ? dT6 : R(1.0 / 6.0) * T;
         unline(dT, T, half * t01, dT6, uy, uyh, p[0][0], p[1][0], p[2][0]);
         {   // x moment 1, halved: (t10, 0, (2/9) t10) / 2
             const R h = half * t10;
@@ -284,10 +283,16 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             p[2][1] = r2 + r1;
         }
         unline(dT6, T6, R(1.0 / 18.0) * t01, R(1.0 / 36.0) * dT, uy, uyh, p[0][2], p[1][2], p[2][2]);
-        const R c6 = S::kFull ? c.T_ref6 : R(kS) * c.T_ref6, c23 = S::kFull ? c.T_ref23 : R(kS) * c.T_ref23;
-        unline(p[0][0], c6 + p[0][0], p[0][1], p[0][2], ux, uxh, dg[7], dg[4], dg[8]);
-        unline(p[1][0], c23 + p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
-        unline(p[2][0], c6 + p[2][0], p[2][1], p[2][2], ux, uxh, dg[6], dg[2], dg[5]);
+        if constexpr (S::kFull) {
+            unline(p[0][0], p[0][0], p[0][1], p[0][2], ux, uxh, dg[7], dg[4], dg[8]);
+            unline(p[1][0], p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
+            unline(p[2][0], p[2][0], p[2][1], p[2][2], ux, uxh, dg[6], dg[2], dg[5]);
+        } else {
+            const R c6 = R(1.0 / 6.0) * T0, c23 = R(2.0 / 3.0) * T0;
+            unline(p[0][0], c6 + p[0][0], p[0][1], p[0][2], ux, uxh, dg[7], dg[4], dg[8]);
+            unline(p[1][0], c23 + p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
+            unline(p[2][0], c6 + p[2][0], p[2][1], p[2][2], ux, uxh, dg[6], dg[2], dg[5]);
+        }
     }
 
     if constexpr (std::is_same<S, StoreF16S>::value) {
@@ -304,7 +309,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
         static_for<9>([&](auto A) {
             constexpr int a = decltype(A)::value;
             S::store_dev(fout, (Idx)a * geo.n + i, df[a], R(w9(a)));
-            S::store_dev(gout, (Idx)a * geo.n + i, dg[a], c.wT[a == 0 ? 0 : (a < 5 ? 1 : 2)]);
+            gout[(Idx)a * geo.n + i] = dg[a];
         });
     }
 }

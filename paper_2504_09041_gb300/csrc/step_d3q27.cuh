@@ -634,19 +634,21 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
     const R drho = z0[0][0], jx = z0[0][1], jy = z0[1][0], jz = z1[0][0];
 
     // energy: T and the first-order moments
-    const R T0 = S::kFull ? c.T_ref : R(kS) * c.T_ref;
-    R dT, gx, gy, gz;
-    {
-        R gs[15];
-#pragma unroll
-        for (int b = 0; b < 15; ++b) gs[b] = g[b];
-        if constexpr (S::kFull) gs[0] -= T0;
-        raw01_g_d3q15(gs, dT, gx, gy, gz);
+    const R T0 = S::kFull ? R(0) : R(kS) * c.T_ref;   // g = dT + T0, as in 2D
+    const R dT = (g[0] + ((g[1] + g[2]) + ((g[3] + g[4]) + (g[5] + g[6]))))
+               + (((g[7] + g[14]) + (g[8] + g[13])) + ((g[9] + g[12]) + (g[10] + g[11])));
+    R gx, gy, gz;
+    {   // along the diagonals (+++), (-++), (+-+), (++-)
+        const R d1 = g[7] - g[14], d2 = g[8] - g[13], d3 = g[9] - g[12], d4 = g[11] - g[10];
+        const R a = d1 + d4, b = d3 - d2;
+        gx = (g[1] - g[2]) + (a + b);
+        gy = (g[3] - g[4]) + (a - b);
+        gz = (g[5] - g[6]) + ((d1 - d4) + (d2 + d3));
     }
-    const R T = T0 + dT, rho = R(kS) + drho;
+    const R T = S::kFull ? dT : T0 + dT, rho = R(kS) + drho;
     check_node_bits(status, rho, T);
     const R irho = recip(rho);
-    const R Fz = c.gbeta * dT, hF = half * Fz;
+    const R Fz = c.gbeta * (S::kFull ? dT - c.T_ref : dT), hF = half * Fz;
     const R pz = jz + hF;                                  // rho u_z (u_x, u_y: no force)
     const R ux = jx * irho, uy = jy * irho, uz = pz * irho;
     const R uxh = half * ux, uyh = half * uy, uzh = half * uz;
@@ -734,20 +736,20 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
     // energy: the moments of collide_g_d3q15_unit as deviations from w T_o
     {
         constexpr double c3 = 2.0 / 9.0;
-        const R rest2 = S::kFull ? two * c.T_ref6 : R(2.0 * kS) * c.T_ref6;
+        const R rest2 = third * T0;
         const R t100 = c.kg[0] * (gx - ux * T), t010 = c.kg[1] * (gy - uy * T), t001 = c.kg[2] * (gz - uz * T);
         const R q100 = t100 + ux * T, q010 = t010 + uy * T, q001 = t001 + uz * T;
         const R xt = ux * t001;
         const R q110 = ux * t010 + uy * q100, q101 = xt + uz * q100, q011 = uy * t001 + uz * q010;
         const R t2 = third * dT;
         const R q200 = t2 + ux * (t100 + q100), q020 = t2 + uy * (t010 + q010), q002 = t2 + uz * (t001 + q001);
-        const R q020f = q020 + rest2;
+        const R q020f = S::kFull ? q020 : q020 + rest2;
         const R q120 = t100 * (R(c3) + uy * uy) + ux * q020f;
-        const R q012 = t010 * (R(c3) + uz * uz) + uy * (q002 + rest2);
-        const R q201 = t001 * (R(c3) + ux * ux) + uz * (q200 + rest2);
+        const R q012 = t010 * (R(c3) + uz * uz) + uy * (S::kFull ? q002 : q002 + rest2);
+        const R q201 = t001 * (R(c3) + ux * ux) + uz * (S::kFull ? q200 : q200 + rest2);
         const R q111 = uy * xt + uz * q110;
         const R Z1 = q012 - ux * (two * q110 - ux * q010);
-        const R Z2 = R(1.0 / 9.0) * dT + uy * (two * Z1 - uy * (third * T));
+        const R Z2 = R(1.0 / 9.0) * dT + uy * (two * Z1 - uy * (S::kFull ? t2 : third * T));
         const R q220 = Z2 + ux * (two * q120 - ux * q020f);
         dg[0] = (dT - q200) - (q020 + q002) + two * q220;
         const R h220 = half * q220, h120 = half * q120, h012 = half * q012, h201 = half * q201;
@@ -796,7 +798,7 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
         });
         static_for<15>([&](auto B) {
             constexpr int b = decltype(B)::value;
-            S::store_dev(gout, (Idx)b * geo.n + i, dg[b], c.wT[b == 0 ? 0 : (b < 7 ? 1 : 2)]);
+            gout[(Idx)b * geo.n + i] = dg[b];
         });
     }
 }
