@@ -30,17 +30,15 @@ static cudaError_t run_adjoint(const void* f_prev, const void* g_prev, const voi
         const int shapes[5][2] = {{0, 0}, {64, 4}, {128, 2}, {32, 4}, {64, 2}};
         const dim3 b(shapes[hc.adj_sync][0], shapes[hc.adj_sync][1], 1);
         const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
-        adjoint_step_d2q9_kernel<S, RT, true><<<grid, b, 0, st>>>(
-            (const T*)f_prev, (const T*)g_prev, (const RT*)mu_in, (RT*)mu_out, geo,
-            make_coeffs<R, 9, 9>(hc), make_coeffs<TapeT<R, RT>, 9, 9>(hc), design_face, grad);
-        return cudaGetLastError();
+        auto kern = unit_rates_2d(hc) ? adjoint_step_d2q9_kernel<S, RT, true, true> : adjoint_step_d2q9_kernel<S, RT, true>;
+        return launch_step_kernel(kern, grid, b, st, (const T*)f_prev, (const T*)g_prev, (const RT*)mu_in, (RT*)mu_out,
+                                  geo, make_coeffs<R, 9, 9>(hc), make_coeffs<TapeT<R, RT>, 9, 9>(hc), design_face, grad);
     }
     const dim3 b(64, 2, 1);
     const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
-    adjoint_step_d2q9_kernel<S, RT><<<grid, b, 0, st>>>(
-        (const T*)f_prev, (const T*)g_prev, (const RT*)mu_in, (RT*)mu_out, geo,
-        make_coeffs<R, 9, 9>(hc), make_coeffs<TapeT<R, RT>, 9, 9>(hc), design_face, grad);
-    return cudaGetLastError();
+    return launch_step_kernel(adjoint_step_d2q9_kernel<S, RT>, grid, b, st, (const T*)f_prev, (const T*)g_prev,
+                              (const RT*)mu_in, (RT*)mu_out, geo, make_coeffs<R, 9, 9>(hc),
+                              make_coeffs<TapeT<R, RT>, 9, 9>(hc), design_face, grad);
 }
 
 cudaError_t launch_adjoint_step_d2q9(int prec, int arith, const void* f_prev, const void* g_prev,

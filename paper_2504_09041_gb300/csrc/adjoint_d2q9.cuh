@@ -408,10 +408,160 @@ __device__ __forceinline__ void collide_forward_tape(const R pf[9], const R pg[9
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The products at the rates lbm_create sets, option A and gravity along y (unit_rates_2d).  A moment
+// relaxed at rate 1 keeps nothing of its pre-collision value, so (1 - omega) makes most adjoints of
+// the central moments zero, and without a force along x the sources reduce to three.  The reduced
+// products below drop exactly those zero terms and keep every other term of the general ones, with the
+// same forward values: the gradient is the same but for the rounding of the sums.
+// ---------------------------------------------------------------------------------------------
+
+// Reverse of the energy relaxation and its forward sweeps: adjoints tb of eta~ -> adjoints inb of the
+// nine links, and of T (Tb), u_x and u_y.  Only eta_10 and eta_01 (and T) carry adjoints back.
+template <class RT, class RF>
+__device__ __forceinline__ void energy_unit_vjp(const RF X[3][3], const RF N[3][3], RF ux, RF uy,
+                                                const Coeffs2D<RF>& c, const RT tb[3][3], RT inb[9],
+                                                RT& uxb, RT& uyb, RT& Tb)
+{
+    const RF* o = c.om_g;
+    const RF one = RF(1), cs2 = RF(1.0 / 3.0);
+    const RF c1 = RF(2.0 / 9.0), c2 = RF(1.0 / 6.0);
+    const RT a22 = tb[2][2];
+    const RT t10b = tb[0][1] + am(tb[2][1], c1);
+    const RT t01b = tb[1][0] + am(tb[1][2], c1);
+    const RT t20b = tb[0][2] + am(a22, c2);
+    const RT t02b = tb[2][0] + am(a22, c2);
+    Tb += am(halve(t20b + t02b), RF(2) * cs2) + tb[0][0];
+    const RT n10b = am(t10b, one - o[1]);
+    const RT n01b = am(t01b, one - o[2]);
+    // y lines: (0, n01, 0), (n10, 0, 0), 0
+    const RT y0 = -RT(am(n01b, uy));
+    uyb -= am(n01b, N[0][0]);
+    const RT X0[3] = {y0 - n01b, y0, y0 + n01b};
+    // x lines (X0_j, n10, 0)
+    const auto un = am(n10b, ux);
+    RT P[3][3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        uxb -= am(n10b, X[j][0]);
+        const RT K0 = X0[j] - un;
+        P[j][0] = K0 - n10b;
+        P[j][1] = K0;
+        P[j][2] = K0 + n10b;
+    }
+    static_for<9>([&](auto I) {
+        constexpr int a = decltype(I)::value;
+        inb[a] = P[e9(a, 1) + 1][e9(a, 0) + 1];
+    });
+}
+
+// Reverse of relax_f_d2q9 and its forward sweeps: adjoints tb of the relaxed deviations -> adjoints inb
+// of the nine links and of drho, irho, u_x, u_y, F_y.  Of the pre-collision moments 20, 02, 11 and 21
+// (through sigma_22) carry adjoints back.
+template <class RT, class RF>
+__device__ __forceinline__ void flow_unit_vjp(const RF X[3][3], const RF D[3][3], RF drho, RF irho, RF ux, RF uy,
+                                              RF Fy, const Coeffs2D<RF>& c, const RT tb[3][3], RT inb[9],
+                                              RT& drhob, RT& irhob, RT& uxb, RT& uyb, RT& Fyb)
+{
+    const RF* o = c.om_f;
+    const RF one = RF(1), two = RF(2), half = RF(0.5), two3 = RF(2.0 / 3.0);
+    const RF third = RF(1.0 / 3.0);
+    const RF Ax = third + ux * ux, By = third + uy * uy, uxuy = ux * uy;
+    const RF D20 = D[0][2], D11 = D[1][1], D21 = D[1][2], D02 = D[2][0];
+    const RF Fyr = Fy * irho;
+    const RF k11 = uxuy + D11, k20 = Ax + D20;
+    const RF k21 = D21 - Ax * uy;
+    const RF D2s = D20 + D02, D2d = D20 - D02;
+    const RF u2s = ux * ux + uy * uy, u2d = ux * ux - uy * uy;
+    const RF T2s = D2s + o[3] * (two3 * drho - u2s - D2s);
+    const RF T2d = D2d - o[4] * (D2d + u2d);
+    const RF T11 = D11 - o[5] * (D11 + uxuy);
+    const RF T20 = half * (T2s + T2d), T02 = half * (T2s - T2d);
+    const RF t11 = uxuy + T11;
+    const RF N = Ax * T02 + By * T20 + T20 * T02 + two * t11 * t11 - Ax * By * drho;
+
+    const RT a11 = tb[1][1], a21 = tb[1][2], a12 = tb[2][1], a22 = tb[2][2];
+    const RT s12b = halve(a12), s21b = halve(a21), s22b = halve(a22);
+    const RT Nb = am(a22, irho);
+    irhob += am(a22, N);
+    RT Axb = am(Nb, T02 - By * drho) + am(a21, uy);
+    RT Byb = am(Nb, T20 - Ax * drho) + am(a12, ux);
+    const RT T02b = tb[2][0] + am(Nb, Ax + T20);
+    const RT T20b = tb[0][2] + am(Nb, By + T02);
+    const RT t11b = am(Nb, RF(4) * t11);
+    drhob -= am(Nb, Ax * By);
+    const RT T11b = a11 + t11b;
+    uxb += am(a12, By);
+    uyb += am(a21, Ax);
+    const RT T2sb = halve(T20b + T02b), T2db = halve(T20b - T02b);
+    RT d11 = am(T11b, one - o[5]);
+    RT uxuyb = t11b - am(T11b, o[5]);
+    const RT D2db = am(T2db, one - o[4]);
+    const auto u2db = am(T2db, o[4]);    // minus the adjoint of u2d; T2sb is minus that of u2s
+    drhob += am(T2sb, two3) + tb[0][0];
+    uxb -= am(T2sb + u2db, two * ux);
+    uyb -= am(T2sb - u2db, two * uy);
+    uyb += tb[1][0];
+    uxb += tb[0][1];
+    Fyb += halve(tb[1][0]);
+    const RT Fyrb = am(s21b, k20) + am(s12b, two * k11) + am(s22b, two * k21);
+    const RT k11b = am(s12b, two * Fyr);
+    const RT k20b = am(s21b, Fyr);
+    const RT d21 = am(s22b, two * Fyr);
+    Axb += k20b - am(d21, uy);
+    uyb -= am(d21, Ax);
+    const RT d20 = D2db + k20b;
+    uxuyb += k11b;
+    d11 += k11b;
+    Fyb += am(Fyrb, irho);
+    irhob += am(Fyrb, Fy);
+    uxb += am(uxuyb, uy) + am(Axb, two * ux);
+    uyb += am(uxuyb, ux) + am(Byb, two * uy);
+
+    // y lines: (0, 0, d02 = -D2db), (0, d11, 0), (d20, d21, 0)
+    RT Xb[3][3];
+    {
+        const RF k0 = D[0][0], k1 = D[1][0], d = k1 + uy * k0;
+        const RT K2 = -D2db;
+        const RT uK = am(K2, uy);
+        const RT Db = -(uK + uK);
+        uyb -= am(K2, d + k1) - am(uK, k0);
+        const RT K0 = am(uK, uy);
+        const RT Q = K0 + K2;
+        Xb[0][0] = Q - Db;
+        Xb[1][0] = K0;
+        Xb[2][0] = Q + Db;
+    }
+    {
+        uyb -= am(d11, D[0][1]);
+        const RT K0 = -RT(am(d11, uy));
+        Xb[0][1] = K0 - d11;
+        Xb[1][1] = K0;
+        Xb[2][1] = K0 + d11;
+    }
+    {
+        uyb -= am(d21, D[0][2]);
+        const RT K0 = d20 - am(d21, uy);
+        Xb[0][2] = K0 - d21;
+        Xb[1][2] = K0;
+        Xb[2][2] = K0 + d21;
+    }
+    RT Pb[3][3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        central_line_vjp(X[j][0], X[j][1], ux, Xb[j][0], Xb[j][1], Xb[j][2], Pb[j][0], Pb[j][1],
+                         Pb[j][2], uxb);
+    static_for<9>([&](auto I) {
+        constexpr int a = decltype(I)::value;
+        inb[a] = Pb[e9(a, 1) + 1][e9(a, 0) + 1];
+    });
+}
+
 // Vector-Jacobian product of the node collision at the forward values tp: adjoints of the
 // post-collision deviations (lf, lg) -> adjoints of the pulled deviations (mf, mg), in RT.
-// kSync: a block-wide barrier between the energy and the flow products (see the kernel).
-template <class RT, class RF, bool kSync = false>
+// kSync: a block-wide barrier between the energy and the flow products (see the kernel).  kUnit: the
+// reduced products.
+template <class RT, class RF, bool kSync = false, bool kUnit = false>
 __device__ __forceinline__ void collide_vjp_d2q9(const CollideTape<RF>& tp, const RT lf[9],
                                                  const RT lg[9], const Coeffs2D<RF>& c, RT mf[9],
                                                  RT mg[9])
@@ -427,25 +577,33 @@ __device__ __forceinline__ void collide_vjp_d2q9(const CollideTape<RF>& tp, cons
         RT Tb[3][3], Nb[3][3];
         unsweeps_vjp(tp.gT, tp.gY, lg, ux, uy, Tb, uxb, uyb);
         RT Tfb = 0;
-        relax_g_d2q9_vjp(c, tp.gT, T, Tb, Nb, Tfb);
+        if constexpr (kUnit) {
+            energy_unit_vjp(tp.gX, tp.gN, ux, uy, c, Tb, mg, uxb, uyb, Tfb);
+        } else {
+            relax_g_d2q9_vjp(c, tp.gT, T, Tb, Nb, Tfb);
+            sweeps_vjp(tp.gX, tp.gN, Nb, ux, uy, mg, uxb, uyb);
+        }
         dTb += Tfb;
-        sweeps_vjp(tp.gX, tp.gN, Nb, ux, uy, mg, uxb, uyb);
     }
     if constexpr (kSync) __syncthreads();
     // flow chain on deviations
     {
         RT Tb[3][3], Db[3][3];
         unsweeps_vjp(tp.fT, tp.fY, lf, ux, uy, Tb, uxb, uyb);
-        relax_f_d2q9_vjp(tp.fD, drho, irho, ux, uy, Fx, Fy, c, Tb, Db, drhob, irhob, uxb, uyb, Fxb, Fyb);
-        sweeps_vjp(tp.fX, tp.fD, Db, ux, uy, mf, uxb, uyb);
+        if constexpr (kUnit) {
+            flow_unit_vjp(tp.fX, tp.fD, drho, irho, ux, uy, Fy, c, Tb, mf, drhob, irhob, uxb, uyb, Fyb);
+        } else {
+            relax_f_d2q9_vjp(tp.fD, drho, irho, ux, uy, Fx, Fy, c, Tb, Db, drhob, irhob, uxb, uyb, Fxb, Fyb);
+            sweeps_vjp(tp.fX, tp.fD, Db, ux, uy, mf, uxb, uyb);
+        }
     }
     // macroscopic fields: u = (j + F/2) irho, irho = 1 / (1 + drho), F = g beta dT along gravity
     const RT jxb = am(uxb, irho), jyb = am(uyb, irho);
-    Fxb += am(uxb, half * irho);
+    if constexpr (!kUnit) Fxb += am(uxb, half * irho);
     Fyb += am(uyb, half * irho);
-    irhob += am(uxb, jx + half * Fx) + am(uyb, jy + half * Fy);
+    irhob += am(uxb, kUnit ? jx : jx + half * Fx) + am(uyb, jy + half * Fy);
     drhob -= am(irhob, irho * irho);
-    const RT Fbb = c.gaxis == 0 ? Fxb : (c.gaxis == 1 ? Fyb : RT(0));
+    const RT Fbb = kUnit || c.gaxis == 1 ? Fyb : (c.gaxis == 0 ? Fxb : RT(0));
     dTb += am(Fbb, c.gbeta);
     static_for<9>([&](auto I) {
         constexpr int a = decltype(I)::value;
@@ -477,6 +635,14 @@ __device__ __forceinline__ int first_fixed_face(const NodeWalls<R>& w)
     return -1;
 }
 
+// Adjoint values, in a kernel that has called wait_previous_step (see ld_step).
+__device__ __forceinline__ dfloat ld_step(const dfloat* p)
+{
+    dfloat v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.hi), "=f"(v.lo) : "l"(p));
+    return v;
+}
+
 // One adjoint step at every node (see the file comment).  mu_in = mu_{k+1}, mu_out = mu_k, both
 // [18][n] in RT (f links 0..8, then g links 0..8); f_prev, g_prev = s_{k-1} in storage format.
 //
@@ -484,7 +650,7 @@ __device__ __forceinline__ int first_fixed_face(const NodeWalls<R>& w)
 // tape, energy VJP, flow VJP), so that they run the same stretch of the long unrolled code at the
 // same time and share its instruction fetches.  Threads beyond the box then compute on a clamped
 // node and store nothing, so every thread reaches every barrier.
-template <class S, class RT, bool kSync = false>
+template <class S, class RT, bool kSync = false, bool kUnit = false>
 __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
     adjoint_step_d2q9_kernel(const typename S::T* __restrict__ f_prev,
                              const typename S::T* __restrict__ g_prev,
@@ -497,6 +663,7 @@ __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     const bool active = x < geo.nx && y < geo.ny;
+    wait_previous_step();
     if (!kSync && !active) return;
     x = min(x, geo.nx - 1);
     y = min(y, geo.ny - 1);
@@ -513,11 +680,11 @@ __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
         R tw;
         const int s = link_source<e9(ob, 0), e9(ob, 1), 0>(geo, w, i, &out, &dir, &tw);
         if (!out) {
-            lf[b] = mu_in[(size_t)b * n + s];
-            lg[b] = mu_in[(size_t)(9 + b) * n + s];
+            lf[b] = ld_step(mu_in + (size_t)b * n + s);
+            lg[b] = ld_step(mu_in + (size_t)(9 + b) * n + s);
         } else {
-            lf[b] = mu_in[(size_t)ob * n + i];
-            const RT m = mu_in[(size_t)(9 + ob) * n + i];
+            lf[b] = ld_step(mu_in + (size_t)ob * n + i);
+            const RT m = ld_step(mu_in + (size_t)(9 + ob) * n + i);
             lg[b] = dir ? -m : m;
         }
     });
@@ -525,12 +692,12 @@ __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
     if constexpr (kSync) __syncthreads();
     // forward pull of p_k from s_{k-1}
     R fr[9], gr[9];
-    pull_d2q9<S, size_t>(f_prev, g_prev, geo, w, i, cr.T_ref, fr, gr);
+    pull_d2q9<S, size_t, kPullAfter>(f_prev, g_prev, geo, w, i, cr.T_ref, fr, gr);
     CollideTape<RF> tape;
     collide_forward_tape(fr, gr, cr, tape);
     if constexpr (kSync) __syncthreads();
     RT mf[9], mg[9];
-    collide_vjp_d2q9<RT, RF, kSync>(tape, lf, lg, c, mf, mg);
+    collide_vjp_d2q9<RT, RF, kSync, kUnit>(tape, lf, lg, c, mf, mg);
     if (!active) return;
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
