@@ -29,20 +29,31 @@ cudaError_t launch_step(int dim, int prec, const void* fin, const void* gin, voi
 // Conversions between storage and double (F32 and F16S store deviations from the rest state;
 // the full value shift + deviation is formed in double).
 // ---------------------------------------------------------------------------------------------
+// float -> double without the conversion instruction, which takes an FP64 pipe slot (16 cycles of an SM
+// per warp, like an addition, even when predicated off), and that pipe bounds these passes.  A
+// subnormal is first scaled by 2^24; infinities and NaN get the wider exponent.
+__device__ __forceinline__ double widen(float v)
+{
+    const bool sub = (__float_as_uint(v) & 0x7f800000u) == 0u;
+    const unsigned x = __float_as_uint(sub ? v * 16777216.0f : v), m = x & 0x7fffffffu;
+    const unsigned bias = sub ? 0x36800000u : (m >= 0x7f800000u ? 0x70000000u : 0x38000000u);
+    const unsigned hi = m == 0u ? 0u : (m >> 3) + bias;
+    return __hiloint2double((int)((x & 0x80000000u) | hi), (int)(x << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
 template <class S> struct Conv;
 template <> struct Conv<StoreF64> {
-    __device__ static double get(const double* p, size_t i, double) { return p[i]; }
+    __device__ static double get(double v, double) { return v; }
     __device__ static void put(double* p, size_t i, double v, double) { p[i] = v; }
 };
 template <> struct Conv<StoreF32> {
-    __device__ static double get(const float* p, size_t i, double s) { return s + (double)p[i]; }
+    __device__ static double get(float v, double s) { return s + widen(v); }
     __device__ static void put(float* p, size_t i, double v, double s) { p[i] = (float)(v - s); }
 };
 template <> struct Conv<StoreF16S> {
-    __device__ static double get(const __half* p, size_t i, double s)
-    {
-        return s + (double)__half2float(p[i]) * (double)StoreF16S::kInvScale;
-    }
+    // (the scale is a power of two: exact in FP32)
+    __device__ static double get(__half v, double s) { return s + widen(__half2float(v) * StoreF16S::kInvScale); }
     __device__ static void put(__half* p, size_t i, double v, double s)
     {
         p[i] = __double2half((v - s) * (double)StoreF16S::kScale);
@@ -52,13 +63,13 @@ template <> struct Conv<StoreF16S> {
 template <int DIM> struct Lat;
 template <> struct Lat<2> {
     static constexpr int QF = 9, QG = 9;
-    __device__ static double wf(int a) { return w9(a); }
-    __device__ static double wg(int a) { return w9(a); }
+    __host__ __device__ static double wf(int a) { return w9(a); }
+    __host__ __device__ static double wg(int a) { return w9(a); }
 };
 template <> struct Lat<3> {
     static constexpr int QF = 27, QG = 15;
-    __device__ static double wf(int a) { return w27(a); }
-    __device__ static double wg(int a) { return w15(a); }
+    __host__ __device__ static double wf(int a) { return w27(a); }
+    __host__ __device__ static double wg(int a) { return w15(a); }
 };
 
 // splitmix64 (Steele, Lea and Flood 2014): output i of the stream whose state starts at seed.
@@ -90,30 +101,52 @@ __global__ void init_kernel(typename S::T* f, typename S::T* g, Geometry geo, do
     }
 }
 
-template <class S, int DIM>
-__global__ void get_pops_kernel(const typename S::T* f, const typename S::T* g, Geometry geo,
-                                double T_ref, double* fo, double* go)
+// Rest values of all planes, flow then energy (w_a and w_b T_ref), formed on the host.
+struct PlaneShifts {
+    double v[42];
+};
+
+// Population I/O: one plane per blockIdx.y, kIoRows elements per thread in flight.  One FP64 operation
+// per element is left for FP32 and FP16 storage (the shift), so reading 160^3 FP32 takes 338 us against 642 with
+// one node of every plane per thread and the conversions on the FP64 pipe (the HBM floor is 303).
+constexpr int kIoRows = 4;
+
+template <class S, int QF>
+__global__ void __launch_bounds__(256)
+    get_pops_kernel(const typename S::T* __restrict__ f, const typename S::T* __restrict__ g, long long n,
+                    PlaneShifts shift, double* __restrict__ fo, double* __restrict__ go)
 {
-    using L = Lat<DIM>;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < geo.n;
-         i += (long long)gridDim.x * blockDim.x) {
-        for (int a = 0; a < L::QF; ++a) fo[(size_t)a * geo.n + i] = Conv<S>::get(f, (size_t)a * geo.n + i, L::wf(a));
-        for (int b = 0; b < L::QG; ++b)
-            go[(size_t)b * geo.n + i] = Conv<S>::get(g, (size_t)b * geo.n + i, L::wg(b) * T_ref);
-    }
+    const int a = blockIdx.y;
+    const typename S::T* src = a < QF ? f + (size_t)a * n : g + (size_t)(a - QF) * n;
+    double* dst = a < QF ? fo + (size_t)a * n : go + (size_t)(a - QF) * n;
+    const double s = shift.v[a];
+    const long long i0 = (long long)blockIdx.x * (256 * kIoRows) + threadIdx.x;
+    typename S::T v[kIoRows];
+#pragma unroll
+    for (int r = 0; r < kIoRows; ++r)
+        if (i0 + 256 * r < n) v[r] = src[i0 + 256 * r];
+#pragma unroll
+    for (int r = 0; r < kIoRows; ++r)
+        if (i0 + 256 * r < n) dst[i0 + 256 * r] = Conv<S>::get(v[r], s);
 }
 
-template <class S, int DIM>
-__global__ void set_pops_kernel(typename S::T* f, typename S::T* g, Geometry geo, double T_ref,
-                                const double* fi, const double* gi)
+template <class S, int QF>
+__global__ void __launch_bounds__(256)
+    set_pops_kernel(typename S::T* __restrict__ f, typename S::T* __restrict__ g, long long n, PlaneShifts shift,
+                    const double* __restrict__ fi, const double* __restrict__ gi)
 {
-    using L = Lat<DIM>;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < geo.n;
-         i += (long long)gridDim.x * blockDim.x) {
-        for (int a = 0; a < L::QF; ++a) Conv<S>::put(f, (size_t)a * geo.n + i, fi[(size_t)a * geo.n + i], L::wf(a));
-        for (int b = 0; b < L::QG; ++b)
-            Conv<S>::put(g, (size_t)b * geo.n + i, gi[(size_t)b * geo.n + i], L::wg(b) * T_ref);
-    }
+    const int a = blockIdx.y;
+    typename S::T* dst = a < QF ? f + (size_t)a * n : g + (size_t)(a - QF) * n;
+    const double* src = a < QF ? fi + (size_t)a * n : gi + (size_t)(a - QF) * n;
+    const double s = shift.v[a];
+    const long long i0 = (long long)blockIdx.x * (256 * kIoRows) + threadIdx.x;
+    double v[kIoRows];
+#pragma unroll
+    for (int r = 0; r < kIoRows; ++r)
+        if (i0 + 256 * r < n) v[r] = src[i0 + 256 * r];
+#pragma unroll
+    for (int r = 0; r < kIoRows; ++r)
+        if (i0 + 256 * r < n) Conv<S>::put(dst, i0 + 256 * r, v[r], s);
 }
 
 // Streamed populations at one node as deviations from the rest state (the pull of the step
@@ -141,42 +174,90 @@ __host__ __device__ constexpr int ev(int a, int d)
     else return e27(a, d);
 }
 
+// Streamed deviations at one node, the pull chosen per warp as in the steps: interior rows without any
+// wall bookkeeping.
+template <class S, int DIM, class Idx>
+__device__ __forceinline__ void pulled_by_warp(const typename S::T* f, const typename S::T* g, const Geometry& geo,
+                                               typename S::R T_ref, int x, int y, int z, int i,
+                                               typename S::R* fo, typename S::R* go)
+{
+    using R = typename S::R;
+    const bool in = x > 0 && x < geo.nx - 1 && y > 0 && y < geo.ny - 1 && (DIM == 2 || (z > 0 && z < geo.nz - 1));
+    if (__all_sync(__activemask(), in)) {
+        if constexpr (DIM == 2) pull_d2q9_interior<S, Idx>(f, g, geo, i, T_ref, fo, go);
+        else pull_d3q27_d3q15_interior<S, Idx>(f, g, geo, i, T_ref, fo, go);
+    } else {
+        const NodeWalls<R> w = node_walls<R>(geo, x, y, z, DIM);
+        if constexpr (DIM == 2) pull_d2q9<S, Idx>(f, g, geo, w, i, T_ref, fo, go);
+        else pull_d3q27_d3q15<S, Idx>(f, g, geo, w, i, T_ref, fo, go);
+    }
+}
+
 // rho, u and T at every node (App. A Step 7, App. B Step 7, Sec. 6.1 force); a null output is not
-// written.  The sums run over the pulled deviations in the storage's register type (FP32 for FP32
-// and FP16 storage, where an FP64 sum made this pass bound by the FP64 pipe) and are promoted to
-// FP64 for the outputs.
-template <class S, int DIM>
-__global__ void fields_kernel(const typename S::T* f, const typename S::T* g, Geometry geo,
-                              HostCoeffs hc, double* rho, double* ux, double* uy, double* uz,
-                              double* Tout)
+// written, and kFlow = false (only T asked for) does not read the flow.  The sums run over the pulled
+// deviations in the storage's register type (FP32 for FP32 and FP16 storage, where an FP64 sum made
+// this pass bound by the FP64 pipe) and are promoted to FP64 for the outputs; there, too, FP64
+// operations are what remains to save: widen() and one reciprocal for the three divisions (for FP32
+// and FP16 storage an ulp of FP64 on values that carry FP32 rounding).  160^3: FP32 133 us against 644 (floor 125), T alone 69
+// against 228; FP64 1067 against 1622.
+template <class S, int DIM, class Idx, bool kFlow>
+__global__ void __launch_bounds__(256)
+    fields_kernel(const typename S::T* f, const typename S::T* g, Geometry geo, double gbeta, double T_ref,
+                  int gaxis, double* rho, double* ux, double* uy, double* uz, double* Tout)
 {
     using R = typename S::R;
     using L = Lat<DIM>;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < geo.n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int z = (int)(i / geo.nxy), rxy = (int)(i - (long long)z * geo.nxy);
-        const int y = rxy / geo.nx, x = rxy - y * geo.nx;
-        R fo[L::QF], go[L::QG];
-        pulled<S, DIM>(f, g, geo, R(hc.T_ref), x, y, z, fo, go);
-        R dT = go[0], drho = fo[0], j[3] = {R(0), R(0), R(0)};
-        static_for<L::QG - 1>([&](auto B) { dT += go[decltype(B)::value + 1]; });
-        static_for<L::QF - 1>([&](auto A) {
-            constexpr int a = decltype(A)::value + 1;
-            drho += fo[a];
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int z = blockIdx.z;
+    if (x >= geo.nx || y >= geo.ny) return;
+    const int i = x + geo.nx * y + geo.nxy * z;
+    R fo[L::QF], go[L::QG];
+    pulled_by_warp<S, DIM, Idx>(f, g, geo, R(T_ref), x, y, z, i, fo, go);
+    R dT = go[0];
+    static_for<L::QG - 1>([&](auto B) { dT += go[decltype(B)::value + 1]; });
+    const double dTd = widen(dT);
+    if (Tout) Tout[i] = T_ref + dTd;
+    if constexpr (kFlow) {
+        R drho, j[3] = {R(0), R(0), R(0)};
+        if constexpr (DIM == 3 && std::is_same<S, StoreF64>::value) {
+            // FP64: over the raw x lines, half the additions
+            R p[3][3][3];
+            xraw_d3q27(fo, p);
+            drho = R(0);
 #pragma unroll
-            for (int d = 0; d < DIM; ++d) {
-                if (ev<DIM>(a, d) == 1) j[d] += fo[a];
-                if (ev<DIM>(a, d) == -1) j[d] -= fo[a];
+            for (int k = 0; k < 3; ++k) {
+                const R layer = (p[k][0][0] + p[k][2][0]) + p[k][1][0];
+                drho += layer;
+                if (k != 1) j[2] += k == 2 ? layer : -layer;
+                j[1] += p[k][2][0] - p[k][0][0];
+                j[0] += (p[k][0][1] + p[k][2][1]) + p[k][1][1];
             }
-        });
-        const double T = hc.T_ref + (double)dT, r = 1.0 + (double)drho;
-        double F[3] = {0.0, 0.0, 0.0};
-        F[hc.gaxis] = hc.gbeta * (double)dT;
+        } else {
+            drho = fo[0];
+            static_for<L::QF - 1>([&](auto A) {
+                constexpr int a = decltype(A)::value + 1;
+                drho += fo[a];
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) {
+                    if (ev<DIM>(a, d) == 1) j[d] += fo[a];
+                    if (ev<DIM>(a, d) == -1) j[d] -= fo[a];
+                }
+            });
+        }
+        const double r = 1.0 + widen(drho);
+        const double hF = 0.5 * (gbeta * dTd);
+        const double ir = recip(r);
+        double* const out[3] = {ux, uy, uz};
         if (rho) rho[i] = r;
-        if (ux) ux[i] = ((double)j[0] + 0.5 * F[0]) / r;
-        if (uy) uy[i] = ((double)j[1] + 0.5 * F[1]) / r;
-        if (uz) uz[i] = ((double)j[2] + 0.5 * F[2]) / r;
-        if (Tout) Tout[i] = T;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (!out[d]) continue;
+            const double m = (d < DIM ? widen(j[d]) : 0.0) + (d == gaxis ? hF : 0.0);
+            const double q = m * ir;
+            // FP64 storage: one correction of the quotient, to the last bit of a division
+            out[d][i] = std::is_same<S, StoreF64>::value ? fma(fma(-q, r, m), ir, q) : q;
+        }
     }
 }
 
@@ -244,24 +325,29 @@ __global__ void __launch_bounds__(256)
     using R = typename S::R;
     using L = Lat<DIM>;
     const int ax = face >> 1, hi = face & 1;
-    const int ext[3] = {geo.nx, geo.ny, geo.nz};
+    const int ext = ax == 0 ? geo.nx : (ax == 1 ? geo.ny : geo.nz);
     NuAcc acc{0.0, -INFINITY, INFINITY, 0x7fffffff, 0x7fffffff};
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_face; t += gridDim.x * blockDim.x) {
-        int c[3];
-        if (ax == 0) { c[1] = t % geo.ny; c[2] = t / geo.ny; }
-        if (ax == 1) { c[0] = t % geo.nx; c[2] = t / geo.nx; }
-        if (ax == 2) { c[0] = t % geo.nx; c[1] = t / geo.nx; }
+        const int n0 = ax == 0 ? geo.ny : geo.nx;   // the faster of the face's two axes
+        const int t1 = DIM == 2 ? 0 : t / n0, t0 = t - t1 * n0;
+        R go[2][L::QG];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {   // both layers' loads in flight together
+            const int c = hi ? ext - 1 - l : l;
+            R fo[L::QF];
+            pulled<S, DIM>(f, g, geo, R(T_ref), ax == 0 ? c : t0, ax == 0 ? t0 : (ax == 1 ? c : t1),
+                           ax == 2 ? c : t1, fo, go[l]);
+        }
         double Tl[2];
+#pragma unroll
         for (int l = 0; l < 2; ++l) {
-            c[ax] = hi ? ext[ax] - 1 - l : l;
-            R fo[L::QF], go[L::QG];
-            pulled<S, DIM>(f, g, geo, R(T_ref), c[0], c[1], c[2], fo, go);
             double s = 0.0;
-            for (int b = 0; b < L::QG; ++b) s += (double)go[b];
+#pragma unroll
+            for (int b = 0; b < L::QG; ++b) s += widen(go[l][b]);
             Tl[l] = T_ref + s;
         }
-        c[ax] = hi ? ext[ax] - 1 : 0;
-        const double Tw = wall_temperature(geo, face, c[0], c[1], c[2]);
+        const int c = hi ? ext - 1 : 0;
+        const double Tw = wall_temperature(geo, face, ax == 0 ? c : t0, ax == 0 ? t0 : (ax == 1 ? c : t1), ax == 2 ? c : t1);
         const double dTdn = -8.0 / 3.0 * Tw + 3.0 * Tl[0] - 1.0 / 3.0 * Tl[1];
         const double nu = scale * dTdn;
         profile[t] = nu;
@@ -323,13 +409,24 @@ cudaError_t launch_init(int dim, int prec, void* f, void* g, const Geometry& geo
     return cudaGetLastError();
 }
 
+template <int DIM>
+static PlaneShifts plane_shifts(double T_ref)
+{
+    using L = Lat<DIM>;
+    PlaneShifts s{};
+    for (int a = 0; a < L::QF; ++a) s.v[a] = L::wf(a);
+    for (int b = 0; b < L::QG; ++b) s.v[L::QF + b] = L::wg(b) * T_ref;
+    return s;
+}
+
 cudaError_t launch_get_pops(int dim, int prec, const void* f, const void* g, const Geometry& geo,
                             double T_ref, double* fo, double* go, cudaStream_t st)
 {
     LBM_DISPATCH(dim, prec, {
         using T = typename S::T;
-        get_pops_kernel<S, D><<<grid_for(geo.n), 256, 0, st>>>((const T*)f, (const T*)g, geo, T_ref,
-                                                               fo, go);
+        const dim3 grid((unsigned)(((long long)geo.n + 256 * kIoRows - 1) / (256 * kIoRows)), Lat<D>::QF + Lat<D>::QG, 1);
+        get_pops_kernel<S, Lat<D>::QF><<<grid, 256, 0, st>>>((const T*)f, (const T*)g, geo.n, plane_shifts<D>(T_ref),
+                                                             fo, go);
     });
     return cudaGetLastError();
 }
@@ -339,7 +436,8 @@ cudaError_t launch_set_pops(int dim, int prec, void* f, void* g, const Geometry&
 {
     LBM_DISPATCH(dim, prec, {
         using T = typename S::T;
-        set_pops_kernel<S, D><<<grid_for(geo.n), 256, 0, st>>>((T*)f, (T*)g, geo, T_ref, fi, gi);
+        const dim3 grid((unsigned)(((long long)geo.n + 256 * kIoRows - 1) / (256 * kIoRows)), Lat<D>::QF + Lat<D>::QG, 1);
+        set_pops_kernel<S, Lat<D>::QF><<<grid, 256, 0, st>>>((T*)f, (T*)g, geo.n, plane_shifts<D>(T_ref), fi, gi);
     });
     return cudaGetLastError();
 }
@@ -348,10 +446,14 @@ cudaError_t launch_fields(int dim, int prec, const void* f, const void* g, const
                           const HostCoeffs& hc, double* rho, double* ux, double* uy, double* uz,
                           double* T, cudaStream_t st)
 {
+    const dim3 b = block_shape(geo, prec, dim), grid = grid_shape(geo, b);
+    const bool flow = rho || ux || uy || uz;
     LBM_DISPATCH(dim, prec, {
         using TT = typename S::T;
-        fields_kernel<S, D><<<grid_for(geo.n), 256, 0, st>>>((const TT*)f, (const TT*)g, geo, hc, rho,
-                                                             ux, uy, uz, T);
+        auto kern = index32(geo, Lat<D>::QF)
+                        ? (flow ? fields_kernel<S, D, unsigned, true> : fields_kernel<S, D, unsigned, false>)
+                        : (flow ? fields_kernel<S, D, size_t, true> : fields_kernel<S, D, size_t, false>);
+        kern<<<grid, b, 0, st>>>((const TT*)f, (const TT*)g, geo, hc.gbeta, hc.T_ref, hc.gaxis, rho, ux, uy, uz, T);
     });
     return cudaGetLastError();
 }

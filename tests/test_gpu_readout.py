@@ -1,0 +1,56 @@
+"""Population and field read-out: every value of the storage type comes back exactly, and each field is
+the same whether it is asked for alone or with the others."""
+import numpy as np
+import pytest
+
+from tests import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2504_09041_gb300 import lbm as L  # noqa: E402
+
+
+@pytest.mark.parametrize("precision,store", [("fp32", np.float32), ("fp16s", np.float16), ("fp64", np.float64)])
+@pytest.mark.parametrize("shape", [(1, 1), (31, 33), (32, 32), (25, 41)])
+def test_populations_round_trip_special_values(precision, store, shape):
+    """With T_ref = 0 the energy planes are stored as they are (FP16 storage: times 2^10), so what comes
+    back is the stored number widened: exact, for zeros, subnormals, infinities and NaN too.  The sizes
+    straddle the 1024 elements of a block."""
+    ny, nx = shape
+    walls = L.Walls((L.LBM_PERIODIC,) * 6, (0,) * 6, 0.0, 0.0, 1)
+    lat = L.Lattice("d2q9", nx, ny, walls=walls, precision=precision)
+    scale = 1024.0 if precision == "fp16s" else 1.0
+    special = np.array([0.0, -0.0, 1e-40, -3e-42, 1.4e-45, 1.1754944e-38, 6e-8, -5.96e-8, 0.1, -1 / 3,
+                        3.4e38, np.inf, -np.inf, np.nan])
+    g = np.resize(special, (9, 1, ny, nx)).astype(np.float64)
+    f, _ = lat.get_populations()
+    lat.set_populations(f, g)
+    fb, gb = lat.get_populations()
+    lat.close()
+    with np.errstate(over="ignore"):
+        want = (g * scale).astype(store).astype(np.float64) / scale
+    np.testing.assert_array_equal(gb, want)
+    np.testing.assert_array_equal(np.signbit(gb[~np.isnan(gb) & (gb != 0)]), np.signbit(want[~np.isnan(gb) & (gb != 0)]))
+    np.testing.assert_array_equal(fb, f)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16s"])
+@pytest.mark.parametrize("lattice,shape", [("d2q9", (1, 9, 70)), ("d3q27", (5, 6, 33)), ("d3q27", (1, 2, 64))])
+def test_fields_alone_equal_fields_together(lattice, shape, precision):
+    nz, ny, nx = shape
+    lat = L.Lattice(lattice, nx, ny, nz, Ra=1e4, precision=precision)
+    f, g = lat.get_populations()
+    lat.set_populations(synth.perturbed(f, 1, 0.05), synth.perturbed(g, 2, 0.05))
+    lat.step(2)
+    names = ("rho", "ux", "uy", "uz", "T")
+    together = lat.fields()
+    for k, name in enumerate(names):
+        out = torch.full(lat.shape, float("nan"), dtype=torch.float64, device="cuda")
+        L.lbm_fields(lat.h, *[out.data_ptr() if i == k else None for i in range(5)], 1)
+        torch.cuda.synchronize()
+        assert torch.equal(out, together[name]), name
+    lat.close()
