@@ -566,7 +566,7 @@ static int build_graph(lbm_s* h, int par)
     int c = par;
     for (int t = 0; t < h->graph_steps && e == cudaSuccess; ++t) {
         e = lbm::launch_step(h->dim, h->prec, h->f[c], h->g[c], h->f[1 - c], h->g[1 - c], h->geo, h->hc,
-                             h->status, dim3(h->block_x, h->block_y, 1), h->capture_stream,
+                             h->status, dim3(h->block_x, h->block_y, 1), c != 0, h->capture_stream,
                              h->tma_rows ? &h->tm[c] : nullptr);
         c = 1 - c;
     }
@@ -602,7 +602,7 @@ int lbm_step(lbm_handle h, long n)
         const int c = h->cur;
         LBM_CK(h, lbm::launch_step(h->dim, h->prec, h->f[c], h->g[c], h->f[1 - c], h->g[1 - c],
                                    h->geo, h->hc, h->status, dim3(h->block_x, h->block_y, 1),
-                                   h->stream, h->tma_rows ? &h->tm[c] : nullptr));
+                                   c != 0, h->stream, h->tma_rows ? &h->tm[c] : nullptr));
         h->cur = 1 - c;
         ++h->steps;
     }
@@ -841,7 +841,8 @@ int lbm_adjoint_step(lbm_handle h, long n_steps, int objective_face, int design_
             cudaError_t e = cudaSuccess;
             for (long r2 = 1; r2 < K && e == cudaSuccess; ++r2)
                 e = lbm::launch_step(h->dim, h->prec, sgf_[s][r2 - 1], sgg_[s][r2 - 1], sgf_[s][r2],
-                                     sgg_[s][r2], h->geo, h->hc, h->status, blk, h->capture_stream);
+                                     sgg_[s][r2], h->geo, h->hc, h->status, blk, (r2 & 1) != 0,
+                                     h->capture_stream);
             const cudaError_t e2 = cudaStreamEndCapture(h->capture_stream, &g);
             if (e == cudaSuccess && e2 == cudaSuccess) e = cudaGraphInstantiate(&seg_exec[s], g, 0);
             if (g) cudaGraphDestroy(g);
@@ -888,7 +889,7 @@ int lbm_adjoint_step(lbm_handle h, long n_steps, int objective_face, int design_
         } else {
             for (long r2 = 1; r2 < hi - lo; ++r2) {
                 ADJ_CK(lbm::launch_step(h->dim, h->prec, sf[r2 - 1], sg[r2 - 1], sgf_[s][r2], sgg_[s][r2],
-                                        h->geo, h->hc, h->status, blk, h->stream));
+                                        h->geo, h->hc, h->status, blk, (r2 & 1) != 0, h->stream));
                 sf[r2] = sgf_[s][r2];
                 sg[r2] = sgg_[s][r2];
             }

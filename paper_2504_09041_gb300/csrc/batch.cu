@@ -55,15 +55,17 @@ __global__ void __launch_bounds__(256, BatchBounds<S>::kMinBlocks)
     batch_step_d2q9_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                            typename S::T* __restrict__ fout, typename S::T* __restrict__ gout,
                            const BatchMember<S>* __restrict__ members, int n_members,
-                           int n_tiles, int tile_x, int tile_y, unsigned* status)
+                           int n_tiles, int tile_x, int tile_y, bool flip, unsigned* status)
 {
     using M = BatchMember<S>;
     __shared__ __align__(16) unsigned char mbuf[sizeof(M)];
     const M& m = *reinterpret_cast<const M*>(mbuf);
     // block b owns the contiguous tile range [t0, t1): equal shares, the first `rem` blocks one more
+    // (flip, alternated from step to step: the shares from the last one, see launch_step)
     const int per = n_tiles / (int)gridDim.x, rem = n_tiles % (int)gridDim.x;
-    const int t0 = (int)blockIdx.x * per + min((int)blockIdx.x, rem);
-    const int t1 = t0 + per + ((int)blockIdx.x < rem ? 1 : 0);
+    const int b = flip ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    const int t0 = b * per + min(b, rem);
+    const int t1 = t0 + per + (b < rem ? 1 : 0);
     // owning member of t0 (every thread reads the same entries, so k is uniform in the block)
     int lo = 0, hi = n_members - 1;
     while (lo < hi) {
@@ -114,12 +116,12 @@ static int resident_blocks(int threads)
 template <class S>
 static cudaError_t launch_batch(const void* fin, const void* gin, void* fout, void* gout,
                                 const void* members, int n_members, int n_tiles, int tile_x,
-                                int tile_y, int grid, unsigned* status, cudaStream_t st)
+                                int tile_y, int grid, bool flip, unsigned* status, cudaStream_t st)
 {
     using T = typename S::T;
     return launch_step_kernel(batch_step_d2q9_kernel<S>, dim3(grid), dim3(tile_x * tile_y), st, (const T*)fin,
                               (const T*)gin, (T*)fout, (T*)gout, (const BatchMember<S>*)members, n_members,
-                              n_tiles, tile_x, tile_y, status);
+                              n_tiles, tile_x, tile_y, flip, status);
 }
 
 }  // namespace lbm
@@ -242,6 +244,7 @@ int upload_table(lbm_batch_s* b)
 }
 
 int max_resident(int prec, int threads);
+size_t elem_bytes(int prec);
 
 // Blocks of one step launch: ctas_per_sm blocks per SM (0 = as many as are resident at once),
 // at most one per tile.
@@ -252,13 +255,14 @@ int grid_of(lbm_batch_s* b)
 }
 
 cudaError_t launch_one(lbm_batch_s* b, const void* fin, const void* gin, void* fout, void* gout,
-                       cudaStream_t st)
+                       bool flip, cudaStream_t st)
 {
     const int grid = grid_of(b);
+    flip = flip && 36.0 * (double)b->total * (double)elem_bytes(b->prec) > 129e6;   // as flip_pays
     switch (b->prec) {
-    case lbm::kF64: return lbm::launch_batch<lbm::StoreF64>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, b->status, st);
-    case lbm::kF32: return lbm::launch_batch<lbm::StoreF32>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, b->status, st);
-    case lbm::kF16S: return lbm::launch_batch<lbm::StoreF16S>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, b->status, st);
+    case lbm::kF64: return lbm::launch_batch<lbm::StoreF64>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, flip, b->status, st);
+    case lbm::kF32: return lbm::launch_batch<lbm::StoreF32>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, flip, b->status, st);
+    case lbm::kF16S: return lbm::launch_batch<lbm::StoreF16S>(fin, gin, fout, gout, b->members, b->count, b->n_tiles, b->tile_x, b->tile_y, grid, flip, b->status, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -293,7 +297,7 @@ int build_batch_graph(lbm_batch_s* b, int par)
     cudaError_t e = cudaSuccess;
     int c = par;
     for (int t = 0; t < b->graph_steps && e == cudaSuccess; ++t) {
-        e = launch_one(b, b->f[c], b->g[c], b->f[1 - c], b->g[1 - c], b->capture_stream);
+        e = launch_one(b, b->f[c], b->g[c], b->f[1 - c], b->g[1 - c], c != 0, b->capture_stream);
         c = 1 - c;
     }
     const cudaError_t e2 = cudaStreamEndCapture(b->capture_stream, &gr);
@@ -437,7 +441,7 @@ int lbm_batch_step(lbm_batch b, long n)
     }
     for (long t = 0; t < n; ++t) {
         const int c = b->cur;
-        B_CK(b, launch_one(b, b->f[c], b->g[c], b->f[1 - c], b->g[1 - c], b->stream));
+        B_CK(b, launch_one(b, b->f[c], b->g[c], b->f[1 - c], b->g[1 - c], c != 0, b->stream));
         b->cur = 1 - c;
         ++b->steps;
     }
@@ -483,7 +487,7 @@ int lbm_batch_tune(lbm_batch b, int trial_steps, int* tile_x, int* tile_y, int* 
             int c = 0;
             for (int t = 0; t < 2 + trial_steps; ++t) {
                 if (t == 2) cudaEventRecord(e0, b->stream);
-                launch_one(b, tf[c], tg[c], tf[1 - c], tg[1 - c], b->stream);
+                launch_one(b, tf[c], tg[c], tf[1 - c], tg[1 - c], c != 0, b->stream);
                 c = 1 - c;
             }
             cudaEventRecord(e1, b->stream);

@@ -71,9 +71,11 @@ bool make_tma_map(CUtensorMap* out, void* base, int elem_bytes, int nx, int ny, 
 
 // block: thread-block shape of the step launch (x-major); block.x == 0 selects the default.
 // tma: tensor maps of fin / gin for the TMA-staged 3D step (FP32 and FP16S), or nullptr.
+// flip: walk the box from its end where flip_pays.  Callers alternate it from step to step; the results
+// are the same.
 cudaError_t launch_step(int dim, int prec, const void* fin, const void* gin, void* fout, void* gout,
                         const Geometry& geo, const HostCoeffs& hc, unsigned* status, dim3 block,
-                        cudaStream_t st, const TmaMaps* tma = nullptr);
+                        bool flip, cudaStream_t st, const TmaMaps* tma = nullptr);
 cudaError_t launch_step_d3q27_tma_f32(const TmaMaps& tm, const void* fin, const void* gin, void* fout,
                                       void* gout, const Geometry& geo, const HostCoeffs& hc,
                                       unsigned* status, cudaStream_t st);
@@ -82,16 +84,16 @@ cudaError_t launch_step_d3q27_tma_f16s(const TmaMaps& tm, const void* fin, const
                                        unsigned* status, cudaStream_t st);
 cudaError_t launch_step_d2q9(int prec, const void* fin, const void* gin, void* fout, void* gout,
                              const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                             dim3 block, cudaStream_t st);
+                             dim3 block, bool flip, cudaStream_t st);
 cudaError_t launch_step_d3q27_f64(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st);
+                                  dim3 block, bool flip, cudaStream_t st);
 cudaError_t launch_step_d3q27_f32(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st);
+                                  dim3 block, bool flip, cudaStream_t st);
 cudaError_t launch_step_d3q27_f16s(const void* fin, const void* gin, void* fout, void* gout,
                                    const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                   dim3 block, cudaStream_t st);
+                                   dim3 block, bool flip, cudaStream_t st);
 
 cudaError_t launch_init(int dim, int prec, void* f, void* g, const Geometry& geo, double T_init,
                         double T_ref, uint64_t seed, double perturb, cudaStream_t st);
@@ -260,6 +262,15 @@ inline int rate_class(const HostCoeffs& h)
 // fastest with every collision (FP32 128^3 106 us against 111 for two rows, 256^3 853 against 862,
 // 32^3 4.1 against 5.7; only the general collision at 256^3 is within 0.2 % either way).
 inline int rows3d_for(const HostCoeffs& h) { return h.rows3d > 0 ? h.rows3d : 1; }
+
+// Both buffers of a box exceed the 129 MB L2.  A step that walks the box in the other direction than the one
+// before it then starts with the rows written last, which are still there: 131 x 93 x 77 FP32 69.4 ->
+// 62.8 us with option B, 128^3 113.5 -> 108.6, 256^3 831 -> 825 (default rates), 2048 x 1024 46.1 -> 44.1.
+// Boxes that fit in L2 as a whole lose a little (64^3 14.5 -> 15.1 us, 1024 x 512 10.0 -> 10.2).
+inline bool flip_pays(const Geometry& g, int q, int prec)
+{
+    return 2.0 * q * (double)g.n * (double)storage_bytes(prec) > 129e6;
+}
 
 inline dim3 grid_shape(const Geometry& g, dim3 b)
 {

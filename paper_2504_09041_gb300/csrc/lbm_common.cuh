@@ -47,6 +47,13 @@ __device__ __forceinline__ __half ld_ro(const __half* p)
     asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
     return __ushort_as_half(v);
 }
+// two neighbouring FP16 values; p on 4 bytes
+__device__ __forceinline__ unsigned ld_ro_pair(const __half* p)
+{
+    unsigned v;
+    asm("ld.global.nc.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ double ld_step(const double* p)
 {
     double v;
@@ -107,14 +114,10 @@ struct StoreF16S {
     __device__ static void store_dev(T* p, size_t i, R dev, R) { p[i] = __float2half_rn(dev * kScale); }
     // a deviation already multiplied by kScale
     __device__ static void store_scaled(T* p, size_t i, R scaled) { p[i] = __float2half_rn(scaled); }
-    // Two deviations converted together with stochastic rounding: each is rounded up or down to a
-    // neighbouring FP16 value with probabilities that make the rounding unbiased, driven by the
-    // caller's random bits (Blackwell's cvt.rs).  Returns (half of d0) | (half of d1) << 16.
-    __device__ static unsigned pack_sr(R d0, R d1, unsigned rbits)
-    {
-        return pack_sr_scaled(d0 * kScale, d1 * kScale, rbits);
-    }
-    // the same for deviations already multiplied by kScale
+    // Two deviations, already multiplied by kScale, converted together with stochastic rounding: each
+    // is rounded up or down to a neighbouring FP16 value with probabilities that make the rounding
+    // unbiased, driven by the caller's random bits (Blackwell's cvt.rs).  Returns
+    // (half of s0) | (half of s1) << 16.
     __device__ static unsigned pack_sr_scaled(R s0, R s1, unsigned rbits)
     {
         unsigned h2;
@@ -381,33 +384,55 @@ __device__ __forceinline__ void static_for(F&& f)
     static_for_impl(f, std::make_integer_sequence<int, N>{});
 }
 
-// Store of one node's 2q deviations (flow planes then energy planes) through F16S storage with
-// stochastic rounding: consecutive values are converted in pairs.  kScaled: df and dg are already
-// multiplied by the storage scale (the seed is still taken from the unscaled values' bits).
-template <int QF, int QG, class Idx, bool kScaled = false>
-__device__ __forceinline__ void store_node_f16s_sr(__half* __restrict__ fout, __half* __restrict__ gout,
-                                                   Idx n, int i, const float* df, const float* dg)
+// One node's q deviations (flow planes then energy planes) rounded to FP16 storage in pairs: word k
+// holds values 2k and 2k + 1.  kStochastic: with the node's random bits (see sr_seed); kScaled: df and
+// dg are already multiplied by the storage scale (the seed is still taken from the unscaled bits).
+template <int QF, int QG, bool kStochastic, bool kScaled>
+__device__ __forceinline__ void pack_node_f16s(int i, const float* df, const float* dg, unsigned h2[(QF + QG) / 2])
 {
     constexpr int Q = QF + QG;
-    const float unscale = kScaled ? StoreF16S::kInvScale : 1.0f;
-    const unsigned seed = sr_seed((unsigned)i, df[0] * unscale, dg[0] * unscale);
-    static_for<(Q + 1) / 2>([&](auto K) {
+    static_assert(Q % 2 == 0, "values are converted in pairs");
+    const float unscale = kScaled ? StoreF16S::kInvScale : 1.0f, scale = kScaled ? 1.0f : StoreF16S::kScale;
+    const unsigned seed = kStochastic ? sr_seed((unsigned)i, df[0] * unscale, dg[0] * unscale) : 0u;
+    static_for<Q / 2>([&](auto K) {
         constexpr int k = decltype(K)::value;
         constexpr int a0 = 2 * k, a1 = 2 * k + 1;
         // value a of the node: flow plane a, or energy plane a - QF (indices kept in range)
         constexpr int f0 = a0 < QF ? a0 : 0, g0 = a0 < QF ? 0 : a0 - QF;
-        constexpr int f1 = a1 < QF ? a1 : 0, g1 = a1 < QF ? 0 : (a1 < Q ? a1 - QF : 0);
+        constexpr int f1 = a1 < QF ? a1 : 0, g1 = a1 < QF ? 0 : a1 - QF;
         const float v0 = a0 < QF ? df[f0] : dg[g0];
-        const float v1 = a1 < Q ? (a1 < QF ? df[f1] : dg[g1]) : 0.0f;
-        const unsigned h2 = kScaled ? StoreF16S::pack_sr_scaled(v0, v1, sr_pair_bits<k>(seed))
-                                    : StoreF16S::pack_sr(v0, v1, sr_pair_bits<k>(seed));
-        const __half h0 = __ushort_as_half((unsigned short)(h2 & 0xffffu));
-        const __half h1 = __ushort_as_half((unsigned short)(h2 >> 16));
-        if (a0 < QF) fout[(Idx)a0 * n + i] = h0;
-        else gout[(Idx)(a0 - QF) * n + i] = h0;
-        if (a1 < QF) fout[(Idx)a1 * n + i] = h1;
-        else if (a1 < Q) gout[(Idx)(a1 - QF) * n + i] = h1;
+        const float v1 = a1 < QF ? df[f1] : dg[g1];
+        if constexpr (kStochastic) {
+            h2[k] = StoreF16S::pack_sr_scaled(v0 * scale, v1 * scale, sr_pair_bits<k>(seed));
+        } else {
+            const __half2 h = __floats2half2_rn(v0 * scale, v1 * scale);
+            h2[k] = *reinterpret_cast<const unsigned*>(&h);
+        }
     });
+}
+
+// Store of one node's packed values.
+template <int QF, int QG, class Idx>
+__device__ __forceinline__ void store_packed_f16s(__half* __restrict__ fout, __half* __restrict__ gout, Idx n, int i,
+                                                  const unsigned h2[(QF + QG) / 2])
+{
+    static_for<QF + QG>([&](auto A) {
+        constexpr int a = decltype(A)::value;
+        const __half h = __ushort_as_half((unsigned short)(a & 1 ? h2[a / 2] >> 16 : h2[a / 2] & 0xffffu));
+        if constexpr (a < QF) fout[(Idx)a * n + i] = h;
+        else gout[(Idx)(a - QF) * n + i] = h;
+    });
+}
+
+// Store of one node's deviations through F16S storage; sr: stochastic rounding.
+template <int QF, int QG, class Idx, bool kScaled = false>
+__device__ __forceinline__ void store_node_f16s(__half* __restrict__ fout, __half* __restrict__ gout, Idx n, int i,
+                                                const float* df, const float* dg, int sr)
+{
+    unsigned h2[(QF + QG) / 2];
+    if (sr) pack_node_f16s<QF, QG, true, kScaled>(i, df, dg, h2);
+    else pack_node_f16s<QF, QG, false, kScaled>(i, df, dg, h2);
+    store_packed_f16s<QF, QG, Idx>(fout, gout, n, i, h2);
 }
 
 // 1 / x to about an ulp: the hardware's approximation y and one step of a power series in its residual

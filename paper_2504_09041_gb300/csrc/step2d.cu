@@ -6,7 +6,7 @@ namespace lbm {
 
 template <class S, bool kUnit>
 static cudaError_t run_as(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
-                          const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
+                          const HostCoeffs& hc, unsigned* status, dim3 block, bool flip, cudaStream_t st)
 {
     using T = typename S::T;
     using R = typename S::R;
@@ -17,27 +17,28 @@ static cudaError_t run_as(const void* fin, const void* gin, void* fout, void* go
     if constexpr (kUnit) c = make_unit_coeffs<R, 2>(hc);
     else c = make_coeffs<R, 9, 9>(hc);
     auto kern = step_index32(geo, 9, hc) ? step_d2q9_kernel<S, unsigned, kUnit> : step_d2q9_kernel<S, size_t, kUnit>;
-    return launch_step_kernel(kern, grid, b, st, (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    return launch_step_kernel(kern, grid, b, st, (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status,
+                              flip);
 }
 
 template <class S>
 static cudaError_t run(const void* fin, const void* gin, void* fout, void* gout, const Geometry& geo,
-                       const HostCoeffs& hc, unsigned* status, dim3 block, cudaStream_t st)
+                       const HostCoeffs& hc, unsigned* status, dim3 block, bool flip, cudaStream_t st)
 {
     if constexpr (has_unit_step<S>::value) {
-        if (unit_rates_2d(hc)) return run_as<S, true>(fin, gin, fout, gout, geo, hc, status, block, st);
+        if (unit_rates_2d(hc)) return run_as<S, true>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
     }
-    return run_as<S, false>(fin, gin, fout, gout, geo, hc, status, block, st);
+    return run_as<S, false>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
 }
 
 cudaError_t launch_step_d2q9(int prec, const void* fin, const void* gin, void* fout, void* gout,
                              const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                             dim3 block, cudaStream_t st)
+                             dim3 block, bool flip, cudaStream_t st)
 {
     switch (prec) {
-    case kF64: return run<StoreF64>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case kF32: return run<StoreF32>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case kF16S: return run<StoreF16S>(fin, gin, fout, gout, geo, hc, status, block, st);
+    case kF64: return run<StoreF64>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case kF32: return run<StoreF32>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case kF16S: return run<StoreF16S>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -11,11 +11,23 @@ namespace lbm {
 template <int kU>
 static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st)
+                                  dim3 block, bool flip, cudaStream_t st)
 {
     using S = StoreF16S;
     using T = typename S::T;
     using R = typename S::R;
+    if constexpr (kU == 3) {
+        // two nodes per thread in large boxes (see the kernel) whose rows start on 4 bytes, unless the
+        // caller chose a launch shape of the one-node kernel
+        const bool aligned = (((uintptr_t)fin | (uintptr_t)gin | (uintptr_t)fout | (uintptr_t)gout) & 3) == 0;
+        if (geo.n >= 6000000 && geo.nx % 2 == 0 && aligned && block.x == 0 && hc.rows3d == 0 && step_index32(geo, 27, hc)) {
+            const int warps = (geo.nx / 2 + 31) / 32;
+            const dim3 pb(warps & 1 ? 32 : 64, 1, 1);
+            step_d3q27_pair_f16s_kernel<unsigned><<<dim3((geo.nx / 2 + pb.x - 1) / pb.x, geo.ny, geo.nz), pb, 0, st>>>(
+                (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, make_unit_coeffs<R, 3>(hc), status, flip);
+            return cudaGetLastError();
+        }
+    }
     const dim3 b = block_shape(geo, kF16S, 3, block);
     const auto c = make_step_coeffs<R, kU>(hc);
     const bool idx32 = step_index32(geo, 27, hc);
@@ -26,20 +38,20 @@ static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fou
                             : step_d3q27_kernel<S, unsigned, 1, kU>;
     dim3 g = grid_shape(geo, b);
     g.y = (g.y + rows - 1) / rows;
-    kern<<<g, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    kern<<<g, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status, flip);
     return cudaGetLastError();
 }
 
 cudaError_t launch_step_d3q27_f16s(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st)
+                                  dim3 block, bool flip, cudaStream_t st)
 {
     switch (rate_class(hc)) {
-    case 3: return launch_plain_f16s<3>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case 2: return launch_plain_f16s<2>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case 1: return launch_plain_f16s<1>(fin, gin, fout, gout, geo, hc, status, block, st);
+    case 3: return launch_plain_f16s<3>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case 2: return launch_plain_f16s<2>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case 1: return launch_plain_f16s<1>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
     }
-    return launch_plain_f16s<0>(fin, gin, fout, gout, geo, hc, status, block, st);
+    return launch_plain_f16s<0>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
 }
 
 template <int TY, int kU>

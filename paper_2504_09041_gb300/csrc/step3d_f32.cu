@@ -11,7 +11,7 @@ namespace lbm {
 template <int kU>
 static cudaError_t launch_plain_f32(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st)
+                                  dim3 block, bool flip, cudaStream_t st)
 {
     using S = StoreF32;
     using T = typename S::T;
@@ -26,20 +26,20 @@ static cudaError_t launch_plain_f32(const void* fin, const void* gin, void* fout
                             : step_d3q27_kernel<S, unsigned, 1, kU>;
     dim3 g = grid_shape(geo, b);
     g.y = (g.y + rows - 1) / rows;
-    kern<<<g, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    kern<<<g, b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status, flip);
     return cudaGetLastError();
 }
 
 cudaError_t launch_step_d3q27_f32(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st)
+                                  dim3 block, bool flip, cudaStream_t st)
 {
     switch (rate_class(hc)) {
     case 3:
-    case 2: return launch_plain_f32<2>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case 1: return launch_plain_f32<1>(fin, gin, fout, gout, geo, hc, status, block, st);
+    case 2: return launch_plain_f32<2>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case 1: return launch_plain_f32<1>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
     }
-    return launch_plain_f32<0>(fin, gin, fout, gout, geo, hc, status, block, st);
+    return launch_plain_f32<0>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
 }
 
 template <int TY, int kU>

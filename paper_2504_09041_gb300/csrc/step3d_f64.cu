@@ -9,7 +9,7 @@ namespace lbm {
 template <int kU>
 static cudaError_t launch_plain_f64(const void* fin, const void* gin, void* fout, void* gout,
                                     const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                    dim3 block, cudaStream_t st)
+                                    dim3 block, bool flip, cudaStream_t st)
 {
     using S = StoreF64;
     using T = typename S::T;
@@ -17,20 +17,20 @@ static cudaError_t launch_plain_f64(const void* fin, const void* gin, void* fout
     const dim3 b = block_shape(geo, kF64, 3, block);
     const auto c = make_step_coeffs<R, kU>(hc);
     auto kern = step_index32(geo, 27, hc) ? step_d3q27_kernel<S, unsigned, 1, kU> : step_d3q27_kernel<S, size_t, 1, kU>;
-    kern<<<grid_shape(geo, b), b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status);
+    kern<<<grid_shape(geo, b), b, 0, st>>>((const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, c, status, flip);
     return cudaGetLastError();
 }
 
 cudaError_t launch_step_d3q27_f64(const void* fin, const void* gin, void* fout, void* gout,
                                   const Geometry& geo, const HostCoeffs& hc, unsigned* status,
-                                  dim3 block, cudaStream_t st)
+                                  dim3 block, bool flip, cudaStream_t st)
 {
     switch (rate_class(hc)) {
-    case 3: return launch_plain_f64<3>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case 2: return launch_plain_f64<2>(fin, gin, fout, gout, geo, hc, status, block, st);
-    case 1: return launch_plain_f64<1>(fin, gin, fout, gout, geo, hc, status, block, st);
+    case 3: return launch_plain_f64<3>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case 2: return launch_plain_f64<2>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
+    case 1: return launch_plain_f64<1>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
     }
-    return launch_plain_f64<0>(fin, gin, fout, gout, geo, hc, status, block, st);
+    return launch_plain_f64<0>(fin, gin, fout, gout, geo, hc, status, block, flip, st);
 }
 
 }  // namespace lbm

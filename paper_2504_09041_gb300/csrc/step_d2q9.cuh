@@ -296,15 +296,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
     }
 
     if constexpr (std::is_same<S, StoreF16S>::value) {
-        if (c.fp16_sr) {
-            store_node_f16s_sr<9, 9, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg);
-        } else {
-            static_for<9>([&](auto A) {
-                constexpr int a = decltype(A)::value;
-                StoreF16S::store_scaled(fout, (Idx)a * geo.n + i, df[a]);
-                StoreF16S::store_scaled(gout, (Idx)a * geo.n + i, dg[a]);
-            });
-        }
+        store_node_f16s<9, 9, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg, c.fp16_sr);
     } else {
         static_for<9>([&](auto A) {
             constexpr int a = decltype(A)::value;
@@ -358,7 +350,7 @@ __device__ __forceinline__ void collide_store_d2q9(typename S::R f[9], typename 
                 constexpr int a = decltype(A)::value;
                 dg[a] = g[a] - R(w9(a)) * c.T_ref;
             });
-            store_node_f16s_sr<9, 9, Idx>(fout, gout, (Idx)geo.n, i, f, dg);
+            store_node_f16s<9, 9, Idx>(fout, gout, (Idx)geo.n, i, f, dg, 1);
             return;
         }
     }
@@ -413,10 +405,10 @@ template <class S, class Idx, bool kUnit = false>
 __global__ void __launch_bounds__(256)
     step_d2q9_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                      typename S::T* __restrict__ fout, typename S::T* __restrict__ gout, Geometry geo,
-                     StepCoeffs2D<S, kUnit> c, unsigned* status)
+                     StepCoeffs2D<S, kUnit> c, unsigned* status, bool flip)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int y = (flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
     wait_previous_step();
     if (x >= geo.nx || y >= geo.ny) return;
     node_step_d2q9<S, Idx, kUnit>(fin, gin, fout, gout, geo, c, status, x, y);

@@ -78,6 +78,41 @@ __device__ __forceinline__ void pull_d3q27_d3q15_interior(const typename S::T* _
     });
 }
 
+// Links of a node on an x wall (or x wrap) that leave the box through x, replaced by the wall
+// rules (or the wrapped source) from global memory; the other links keep their staged values.
+template <class S, class Idx, int kPull>
+__device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict__ fin,
+                                                 const typename S::T* __restrict__ gin,
+                                                 const Geometry& geo, int x, int y, int z, int i,
+                                                 typename S::R T_ref, typename S::R f[27],
+                                                 typename S::R g[15])
+{
+    using R = typename S::R;
+    const NodeWalls<R> w = node_walls_x<R>(geo, x, y, z);
+    static_for<27>([&](auto A) {
+        constexpr int a = decltype(A)::value;
+        constexpr int ex = e27(a, 0);
+        if constexpr (ex != 0) {
+            const bool leaves = ex == 1 ? x == 0 : x == geo.nx - 1;
+            if (leaves) {
+                constexpr int o = opp27(a);
+                bool out, dir;
+                R tw;
+                const int s = link_source<ex, e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
+                const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
+                f[a] = load_link<S, kPull>(fin, off, R(w27(a)));
+                constexpr int b = g15_of_27(a);
+                if constexpr (b >= 0) {
+                    constexpr int ob = opp15(b);
+                    const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
+                    const R gv = load_link<S, kPull>(gin, og, R(w15(b)) * T_ref);
+                    g[b] = dir ? anti_bounce<S, kPull>(gv, w15(b), tw, T_ref) : gv;
+                }
+            }
+        }
+    });
+}
+
 // Flow collision (reading R6 of the oracle notes) on the deviations: D[c][b][a] = kappa_abc - K_abc
 // on entry, kappa~_abc - K_abc on exit.  Rate slots follow the moment order of Sec. 5.2; slot 7
 // relaxes the trace (bulk), slots 8 and 9 the deviators kappa_200 - kappa_020, kappa_200 - kappa_002.
@@ -572,7 +607,7 @@ __device__ __forceinline__ void raw01_g_d3q15(const R g[15], R& r000, R& r100, R
     r001 = (g[5] - g[6]) + Cz;
 }
 
-// Both collisions and the store of one node at the rates lbm_create sets, option A and gravity along
+// Both collisions of one node at the rates lbm_create sets, option A and gravity along
 // z (rate_class 3, checked by the host), from the stored numbers in f and g (raw); the 3D
 // counterpart of collide_store_d2q9_unit, see there.  Of the flow's moments only those enter that
 // relax with a rate of their own (rho, j and order 2) or that the force multiplies (orders 0-1 in z, up
@@ -582,13 +617,11 @@ __device__ __forceinline__ void raw01_g_d3q15(const R g[15], R& r000, R& r100, R
 // per node against 867 with the two reduced collisions above alone: 128^3 in FP64 2.33 ms against
 // 3.36 per step; FP16 storage issues 1,012 instructions against 1,249: 81 us against 95 at 128^3, where
 // half of it comes from L2.
-template <class S, class Idx>
-__device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[27], const typename S::R g[15],
-                                                         typename S::T* __restrict__ fout,
-                                                         typename S::T* __restrict__ gout,
-                                                         const Geometry& geo,
-                                                         const UnitCoeffs<typename S::R>& c,
-                                                         unsigned* status, int i)
+// df, dg: the post-collision deviations (FP64 energy: the populations), in storage units.
+template <class S>
+__device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], const typename S::R g[15],
+                                                   const UnitCoeffs<typename S::R>& c, unsigned* status,
+                                                   typename S::R df[27], typename S::R dg[15])
 {
     using R = typename S::R;
     constexpr double kS = S::kUnits;
@@ -718,7 +751,6 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
         unline(x220, R(kS / 36.0) + x220, x221, x222, uz, uzh, p[0][2][2], p[1][2][2], p[2][2][2]);
     }
     // along y, then x; wz and wy are the rest weights of the links already formed
-    R df[27], dg[15];
     static_for<3>([&](auto K) {
         constexpr int k = decltype(K)::value;
         constexpr double wz = kS * (k == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
@@ -778,19 +810,21 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
         dg[14] = D0 - D1;
     }
 
+}
+
+template <class S, class Idx>
+__device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[27], const typename S::R g[15],
+                                                         typename S::T* __restrict__ fout,
+                                                         typename S::T* __restrict__ gout,
+                                                         const Geometry& geo,
+                                                         const UnitCoeffs<typename S::R>& c,
+                                                         unsigned* status, int i)
+{
+    using R = typename S::R;
+    R df[27], dg[15];
+    collide_d3q27_unit<S>(f, g, c, status, df, dg);
     if constexpr (std::is_same<S, StoreF16S>::value) {
-        if (c.fp16_sr) {
-            store_node_f16s_sr<27, 15, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg);
-        } else {
-            static_for<27>([&](auto A) {
-                constexpr int a = decltype(A)::value;
-                StoreF16S::store_scaled(fout, (Idx)a * geo.n + i, df[a]);
-            });
-            static_for<15>([&](auto B) {
-                constexpr int b = decltype(B)::value;
-                StoreF16S::store_scaled(gout, (Idx)b * geo.n + i, dg[b]);
-            });
-        }
+        store_node_f16s<27, 15, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg, c.fp16_sr);
     } else {
         static_for<27>([&](auto A) {
             constexpr int a = decltype(A)::value;
@@ -926,7 +960,7 @@ __device__ __forceinline__ void collide_store_d3q27(typename S::R f[27], typenam
 
     if constexpr (kF16) {
         if (c.fp16_sr) {
-            store_node_f16s_sr<27, 15, Idx, true>(fout, gout, (Idx)geo.n, i, f, g);
+            store_node_f16s<27, 15, Idx, true>(fout, gout, (Idx)geo.n, i, f, g, 1);
         } else {
             static_for<27>([&](auto A) {
                 constexpr int a = decltype(A)::value;
@@ -966,11 +1000,11 @@ template <class S, class Idx, int kRows = 1, int kRates = 0>
 __global__ void __maxnreg__(LBM_MAXREG3D)
     step_d3q27_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
                       typename S::T* __restrict__ fout, typename S::T* __restrict__ gout,
-                      Geometry geo, StepCoeffs3D<S, kRates> c, unsigned* status)
+                      Geometry geo, StepCoeffs3D<S, kRates> c, unsigned* status, bool flip)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * kRows;
-    const int z = blockIdx.z;
+    const int y0 = ((flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y) * kRows;
+    const int z = flip ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
     if (x >= geo.nx) return;
 #pragma unroll 1
     for (int r = 0; r < kRows; ++r) {
@@ -978,6 +1012,108 @@ __global__ void __maxnreg__(LBM_MAXREG3D)
         if (y >= geo.ny) return;
         node_step_d3q27<S, Idx, kRates>(fin, gin, fout, gout, geo, c, status, x, y, z);
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// FP16 storage, reduced collision: two x-adjacent nodes per thread
+// ---------------------------------------------------------------------------------------------
+
+#ifndef LBM_MAXREG3D_PAIR
+#define LBM_MAXREG3D_PAIR 96
+#endif
+
+__device__ __forceinline__ __half low_half(unsigned w) { return __ushort_as_half((unsigned short)(w & 0xffffu)); }
+__device__ __forceinline__ __half high_half(unsigned w) { return __ushort_as_half((unsigned short)(w >> 16)); }
+
+// Both collisions of one node of a pair, rounded to packed storage.
+__device__ __forceinline__ void pair_node(const float f[27], const float g[15], const UnitCoeffs<float>& c,
+                                          unsigned* status, int i, unsigned h2[21])
+{
+    float df[27], dg[15];
+    collide_d3q27_unit<StoreF16S>(f, g, c, status, df, dg);
+    if (c.fp16_sr) pack_node_f16s<27, 15, true, true>(i, df, dg, h2);
+    else pack_node_f16s<27, 15, false, true>(i, df, dg, h2);
+}
+
+// 32 consecutive FP16 values are only 64 bytes, so one node per thread makes twice the memory requests
+// per byte of FP32, and at 256^3 the step ran at the FP32 step's node rate with DRAM 42 % busy and
+// more warps or fewer instructions no help.  Here a thread updates nodes x0, x0 + 1 (x0 even): links
+// without an x component load, and all links store, 32 bits at once; links along x are two 16-bit
+// loads, the second a hit in L1.  The second node waits as packed halves (hold) while the first
+// is computed, so registers stay near one node's (96, no spills; 80 and 112 measured slower).
+// 256^3: 798 -> 677 us per step (26 % -> 31 % of HBM bandwidth reading and writing each value once);
+// where L2 serves part of the loads the one-node kernel is faster (128^3 79 against 96 us, 160^3 166
+// against 207), so boxes take this one from 6 million nodes on (192^3: 302 against 325).
+// Needs an even nx (then rows and planes start on 4 bytes).  The results are bitwise those of the
+// one-node kernel.
+template <class Idx>
+__global__ void __maxnreg__(LBM_MAXREG3D_PAIR)
+    step_d3q27_pair_f16s_kernel(const __half* __restrict__ fin, const __half* __restrict__ gin,
+                                __half* __restrict__ fout, __half* __restrict__ gout, Geometry geo,
+                                UnitCoeffs<float> c, unsigned* status, bool flip)
+{
+    using S = StoreF16S;
+    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    // the two slices of wall rows, whose blocks take longest, first
+    const int nz = geo.nz, bz = blockIdx.z;
+    const int z = bz == 0 ? (flip ? nz - 1 : 0) : (bz == 1 ? (flip ? 0 : nz - 1) : (flip ? nz - bz : bz - 1));
+    const int y = flip ? geo.ny - 1 - blockIdx.y : blockIdx.y;
+    if (x >= geo.nx) return;
+    const int i = x + geo.nx * y + geo.nxy * z;
+    const Idx n = (Idx)geo.n;
+    const bool yz_in = y > 0 && y < geo.ny - 1 && z > 0 && z < geo.nz - 1;   // uniform in the block
+    unsigned out0[21];
+    float f[27], g[15];
+    if (yz_in) {
+        unsigned hold[21];
+        {
+            // word a: the pair's values on link a (first node low)
+            unsigned w[42];
+            // an x link that would leave the row reads its partner's place instead (fix_x_edge_d3q27
+            // replaces it): the row behind the last one may end the buffer
+            const int lo = x > 0 ? i - 1 : i, hi = x + 2 < geo.nx ? i + 2 : i + 1;
+            static_for<42>([&](auto A) {
+                constexpr int a = decltype(A)::value;
+                constexpr int l = a < 27 ? a : (a - 27 < 7 ? a - 27 : a - 27 + 12);   // D3Q27 link
+                constexpr int ex = e27(l, 0);
+                const __half* p = a < 27 ? fin + (Idx)a * n : gin + (Idx)(a < 27 ? 0 : a - 27) * n;
+                const int row = e27(l, 1) * geo.nx + e27(l, 2) * geo.nxy;
+                if constexpr (ex == 0) {
+                    w[a] = ld_ro_pair(p + (i - row));
+                } else {
+                    const int s0 = (ex == 1 ? lo : i + 1) - row, s1 = (ex == 1 ? i : hi) - row;
+                    w[a] = (unsigned)__half_as_ushort(ld_ro(p + s0)) | (unsigned)__half_as_ushort(ld_ro(p + s1)) << 16;
+                }
+            });
+            static_for<21>([&](auto K) {
+                constexpr int k = decltype(K)::value;
+                hold[k] = __byte_perm(w[2 * k], w[2 * k + 1], 0x7632);
+            });
+            static_for<27>([&](auto A) { f[decltype(A)::value] = S::raw(low_half(w[decltype(A)::value])); });
+            static_for<15>([&](auto B) { g[decltype(B)::value] = S::raw(low_half(w[27 + decltype(B)::value])); });
+        }
+        if (x == 0) fix_x_edge_d3q27<S, Idx, kPullRaw>(fin, gin, geo, x, y, z, i, c.T_ref, f, g);
+        pair_node(f, g, c, status, i, out0);
+        static_for<42>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            const __half h = (a & 1) ? high_half(hold[a / 2]) : low_half(hold[a / 2]);
+            if constexpr (a < 27) f[a] = S::raw(h);
+            else g[a - 27] = S::raw(h);
+        });
+        if (x + 2 == geo.nx) fix_x_edge_d3q27<S, Idx, kPullRaw>(fin, gin, geo, x + 1, y, z, i + 1, c.T_ref, f, g);
+    } else {
+        pull_d3q27_d3q15<S, Idx, kPullRaw>(fin, gin, geo, node_walls<float>(geo, x, y, z, 3), i, c.T_ref, f, g);
+        pair_node(f, g, c, status, i, out0);
+        pull_d3q27_d3q15<S, Idx, kPullRaw>(fin, gin, geo, node_walls<float>(geo, x + 1, y, z, 3), i + 1, c.T_ref, f, g);
+    }
+    unsigned out1[21];
+    pair_node(f, g, c, status, i + 1, out1);
+    static_for<42>([&](auto A) {
+        constexpr int a = decltype(A)::value;
+        const unsigned v = __byte_perm(out0[a / 2], out1[a / 2], (a & 1) ? 0x7632 : 0x5410);
+        __half* p = a < 27 ? fout + (Idx)a * n : gout + (Idx)(a < 27 ? 0 : a - 27) * n;
+        *reinterpret_cast<unsigned*>(p + i) = v;
+    });
 }
 
 }  // namespace lbm

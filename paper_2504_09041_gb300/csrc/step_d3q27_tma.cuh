@@ -131,41 +131,6 @@ __device__ __forceinline__ void tma_issue_tile(const CUtensorMap* mf, const CUte
     });
 }
 
-// Links of a node on an x wall (or x wrap) that leave the box through x, replaced by the wall
-// rules (or the wrapped source) from global memory; the other links keep their staged values.
-template <class S, class Idx, int kPull>
-__device__ __forceinline__ void fix_x_edge_d3q27(const typename S::T* __restrict__ fin,
-                                                 const typename S::T* __restrict__ gin,
-                                                 const Geometry& geo, int x, int y, int z, int i,
-                                                 typename S::R T_ref, typename S::R f[27],
-                                                 typename S::R g[15])
-{
-    using R = typename S::R;
-    const NodeWalls<R> w = node_walls_x<R>(geo, x, y, z);
-    static_for<27>([&](auto A) {
-        constexpr int a = decltype(A)::value;
-        constexpr int ex = e27(a, 0);
-        if constexpr (ex != 0) {
-            const bool leaves = ex == 1 ? x == 0 : x == geo.nx - 1;
-            if (leaves) {
-                constexpr int o = opp27(a);
-                bool out, dir;
-                R tw;
-                const int s = link_source<ex, e27(a, 1), e27(a, 2)>(geo, w, i, &out, &dir, &tw);
-                const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-                f[a] = load_link<S, kPull>(fin, off, R(w27(a)));
-                constexpr int b = g15_of_27(a);
-                if constexpr (b >= 0) {
-                    constexpr int ob = opp15(b);
-                    const Idx og = out ? (Idx)ob * geo.n + i : (Idx)b * geo.n + s;
-                    const R gv = load_link<S, kPull>(gin, og, R(w15(b)) * T_ref);
-                    g[b] = dir ? anti_bounce<S, kPull>(gv, w15(b), tw, T_ref) : gv;
-                }
-            }
-        }
-    });
-}
-
 // Block: TY rows of 64 consumer threads (one node each) and one producer warp whose first lane
 // issues the tensor copies.  The tiles of a block are a contiguous range of the tile list (x
 // fastest, then y, then z), walked with incrementally updated coordinates.  Stage s of the

@@ -85,3 +85,26 @@ def test_reduced_step_equals_general_collision(dim, kind, shape, precision):
         else:
             assert diff <= STEP_TOL[precision]
     assert np.abs(out[0][0] - start[0]).max() > 0
+
+
+@pytest.mark.parametrize("kind,shape,stochastic", [("cavity", (150, 160, 254), 1), ("mixed3d", (97, 251, 258), 0),
+                                                   ("periodic", (61, 1541, 64), 1), ("cavity", (2, 3, 1000002), 1),
+                                                   ("mixed3d", (1000, 3001, 2), 1)])
+def test_fp16s_node_pairs_equal_single_nodes(kind, shape, stochastic):
+    """Boxes of six million nodes and more with an even nx update two nodes per thread; rows3d = 1 selects
+    the one-node kernel.  Bitwise equal, walls and periodic ends included, after steps that move
+    values through each of them; an odd number of steps, so that both walking directions run."""
+    nz, ny, nx = shape
+    states = []
+    for rows in (0, 1):
+        gpu = L.Lattice("d3q27", nx, ny, nz, Ra=1e4, walls=walls_pair(kind, 3, seed=5, perturb=0.05)[0],
+                        precision="fp16s")
+        gpu.set_param("fp16_stochastic", stochastic)
+        gpu.set_param("gbeta", 3e-3)
+        if rows:
+            gpu.set_param("rows3d", rows)
+        gpu.step(5)
+        gpu.sync()
+        states.append(gpu.get_state()[64:])
+        gpu.close()
+    assert np.array_equal(states[0], states[1])
