@@ -47,6 +47,8 @@ struct lbm_s {
     double* nu_profile = nullptr;   // max face nodes
     double* nu_scratch = nullptr;   // block partials
     double* nu_result = nullptr;    // 5 doubles
+    double nu_host[5] = {};         // the same on the host, written by the kernel where host_writes()
+    bool host_writes = false;
     unsigned* ticket = nullptr;
     unsigned* status = nullptr;
     cudaStream_t stream = nullptr;
@@ -342,6 +344,8 @@ int lbm_create(int lattice, int nx, int ny, int nz, double Ra, double Pr, double
     h->nu = P.nu;
     h->alpha = P.alpha;
     h->hc = P.hc;
+
+    h->host_writes = lbm::host_writes();
 
     // Device memory.
     const size_t sb = lbm::storage_bytes(prec);
@@ -656,7 +660,7 @@ int lbm_fields(lbm_handle h, double* rho, double* ux, double* uy, double* uz, do
     return LBM_OK;
 }
 
-static int nusselt_common(lbm_s* h, int face)
+static int nusselt_common(lbm_s* h, int face, double* profile, double* result)
 {
     if (face < 0 || face >= 2 * h->dim) return fail(h, LBM_EINVAL, "face %d is not a face of this box", face);
     if (h->geo.kind[face] != LBM_WALL_FIXED_T) return fail(h, LBM_EINVAL, "face %d is not a fixed-temperature wall", face);
@@ -664,8 +668,8 @@ static int nusselt_common(lbm_s* h, int face)
     if (ext[face / 2] < 2) return fail(h, LBM_EINVAL, "fewer than two node layers normal to face %d", face);
     const double s = h->geo.T_wall[face] >= h->hc.T_ref ? 1.0 : -1.0;
     LBM_CK(h, lbm::launch_nusselt(h->dim, h->prec, h->f[h->cur], h->g[h->cur], h->geo, h->hc, face,
-                                  -s * h->L / h->dT, h->nu_profile, h->nu_scratch, h->ticket,
-                                  h->nu_result, h->stream));
+                                  -s * h->L / h->dT, profile, h->nu_scratch, h->ticket, result,
+                                  h->stream));
     return LBM_OK;
 }
 
@@ -673,10 +677,11 @@ int lbm_nusselt(lbm_handle h, int face, double* mean, double* nu_max, double* nu
                 int* j_min)
 {
     if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
-    int rc = nusselt_common(h, face);
+    double* const r = h->nu_host;
+    int rc = nusselt_common(h, face, h->nu_profile, h->host_writes ? r : h->nu_result);
     if (rc) return rc;
-    double r[5];
-    LBM_CK(h, cudaMemcpyAsync(r, h->nu_result, sizeof r, cudaMemcpyDeviceToHost, h->stream));
+    if (!h->host_writes)
+        LBM_CK(h, cudaMemcpyAsync(r, h->nu_result, sizeof h->nu_host, cudaMemcpyDeviceToHost, h->stream));
     LBM_CK(h, cudaStreamSynchronize(h->stream));
     const long n = face_nodes(h, face);
     if (mean) *mean = r[0] / (double)n;
@@ -690,11 +695,13 @@ int lbm_nusselt(lbm_handle h, int face, double* mean, double* nu_max, double* nu
 int lbm_nusselt_profile(lbm_handle h, int face, double* nu, long n, int device_ptrs)
 {
     if (!h || !nu) return fail(h, LBM_EINVAL, "handle or output is NULL");
-    int rc = nusselt_common(h, face);
+    // the face is checked before its length is, and the length before the kernel writes n values
+    const bool fits = face >= 0 && face < 2 * h->dim && n == face_nodes(h, face);
+    int rc = nusselt_common(h, face, device_ptrs && fits ? nu : h->nu_profile, h->nu_result);
     if (rc) return rc;
-    if (n != face_nodes(h, face)) return fail(h, LBM_EINVAL, "face %d has %ld nodes, not %ld", face, face_nodes(h, face), n);
-    LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double),
-                              device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+    if (!fits) return fail(h, LBM_EINVAL, "face %d has %ld nodes, not %ld", face, face_nodes(h, face), n);
+    if (!device_ptrs)
+        LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     LBM_CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }

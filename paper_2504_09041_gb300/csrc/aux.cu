@@ -1,4 +1,6 @@
 // aux.cu -- initial state, macroscopic fields, population I/O and the wall Nusselt reduction.
+#include <algorithm>
+
 #include "kernels.h"
 #include "step_d2q9.cuh"
 #include "step_d3q27.cuh"
@@ -266,12 +268,37 @@ __global__ void __launch_bounds__(256)
 // Wall Nusselt number (Sec. 6.1): dT/dn = -8/3 T_w + 3 T_1 - 1/3 T_2 from the wall and the first
 // two node layers; Nu = scale * dT/dn with scale = -s L / dT.  One thread per wall node, then
 // FP64 warp-shuffle reductions of (sum, max with index, min with index), per-block partials and a
-// final pass by the last block to finish (deterministic order, ties to the lowest index).
+// final pass by the last block to finish (deterministic order, ties to the lowest index); a face of
+// one block needs neither.
 // ---------------------------------------------------------------------------------------------
+// Extrema are kept as integer keys in the order of the values: an FP64 comparison takes an FP64 pipe slot,
+// and the reductions are chains of them.  A NaN counts for neither (its keys lie beyond the infinities').
 struct NuAcc {
-    double sum, mx, mn;
+    double sum;
+    long long mx, mn;
     int imx, imn;
 };
+
+__device__ __forceinline__ long long nu_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double nu_value(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+// the neutral element: sum 0, max -inf, min +inf at no node
+__device__ __forceinline__ NuAcc nu_none()
+{
+    return NuAcc{0.0, nu_key(-INFINITY), nu_key(INFINITY), 0x7fffffff, 0x7fffffff};
+}
+__device__ __forceinline__ NuAcc nu_node(double nu, int t)
+{
+    const bool nan = (__double_as_longlong(nu) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+    const long long k = nu_key(nu);
+    return NuAcc{nu, nan ? nu_key(-INFINITY) : k, nan ? nu_key(INFINITY) : k, nan ? 0x7fffffff : t, nan ? 0x7fffffff : t};
+}
 
 __device__ __forceinline__ void nu_merge(NuAcc& a, const NuAcc& b)
 {
@@ -303,12 +330,21 @@ __device__ __forceinline__ NuAcc nu_block_reduce(NuAcc a)
     if (lane == 0) warp_part[wid] = a;
     __syncthreads();
     if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        NuAcc b = lane < nw ? warp_part[lane]
-                            : NuAcc{0.0, -INFINITY, INFINITY, 0x7fffffff, 0x7fffffff};
-        a = nu_warp_reduce(b);
+        const int nw = blockDim.x >> 5;
+        // few warps: merged one after the other, no second tree
+        if (nw <= 4) {
+            for (int k = 1; k < nw; ++k) nu_merge(a, warp_part[k]);
+        } else {
+            a = nu_warp_reduce(lane < nw ? warp_part[lane] : nu_none());
+        }
     }
     return a;
+}
+
+// The five result numbers {sum, max, argmax, min, argmin}.
+__device__ __forceinline__ void nu_write(double* r, const NuAcc& a)
+{
+    r[0] = a.sum; r[1] = nu_value(a.mx); r[2] = (double)a.imx; r[3] = nu_value(a.mn); r[4] = (double)a.imn;
 }
 
 size_t nusselt_scratch_doubles(long n_face)
@@ -327,7 +363,7 @@ __global__ void __launch_bounds__(256)
     using L = Lat<DIM>;
     const int ax = face >> 1, hi = face & 1;
     const int ext = ax == 0 ? geo.nx : (ax == 1 ? geo.ny : geo.nz);
-    NuAcc acc{0.0, -INFINITY, INFINITY, 0x7fffffff, 0x7fffffff};
+    NuAcc acc = nu_none();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_face; t += gridDim.x * blockDim.x) {
         const int n0 = ax == 0 ? geo.ny : geo.nx;   // the faster of the face's two axes
         const int t1 = DIM == 2 ? 0 : t / n0, t0 = t - t1 * n0;
@@ -352,13 +388,16 @@ __global__ void __launch_bounds__(256)
         const double dTdn = -8.0 / 3.0 * Tw + 3.0 * Tl[0] - 1.0 / 3.0 * Tl[1];
         const double nu = scale * dTdn;
         profile[t] = nu;
-        nu_merge(acc, NuAcc{nu, nu, nu, t, t});
+        nu_merge(acc, nu_node(nu, t));
     }
     acc = nu_block_reduce(acc);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) nu_write(result, acc);
+        return;
+    }
     __shared__ bool last;
     if (threadIdx.x == 0) {
-        double* p = partials + 5 * blockIdx.x;
-        p[0] = acc.sum; p[1] = acc.mx; p[2] = (double)acc.imx; p[3] = acc.mn; p[4] = (double)acc.imn;
+        nu_write(partials + 5 * blockIdx.x, acc);
         __threadfence();
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
@@ -366,15 +405,14 @@ __global__ void __launch_bounds__(256)
     if (!last) return;
     __threadfence();
     // Final pass: thread k takes partials k, k + blockDim, ... in order, then a block reduction.
-    NuAcc tot{0.0, -INFINITY, INFINITY, 0x7fffffff, 0x7fffffff};
+    NuAcc tot = nu_none();
     for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
         const volatile double* p = partials + 5 * k;
-        nu_merge(tot, NuAcc{p[0], p[1], p[3], (int)p[2], (int)p[4]});
+        nu_merge(tot, NuAcc{p[0], nu_key(p[1]), nu_key(p[3]), (int)p[2], (int)p[4]});
     }
     tot = nu_block_reduce(tot);
     if (threadIdx.x == 0) {
-        result[0] = tot.sum; result[1] = tot.mx; result[2] = (double)tot.imx;
-        result[3] = tot.mn; result[4] = (double)tot.imn;
+        nu_write(result, tot);
         *ticket = 0u;
     }
 }
@@ -459,6 +497,18 @@ cudaError_t launch_fields(int dim, int prec, const void* f, const void* g, const
     return cudaGetLastError();
 }
 
+bool host_writes()
+{
+    int dev = 0, v = 0, w = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&w, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return v != 0 && w != 0;
+}
+
 cudaError_t launch_nusselt(int dim, int prec, const void* f, const void* g, const Geometry& geo,
                            const HostCoeffs& hc, int face, double scale, double* profile,
                            double* scratch, unsigned* ticket, double* result, cudaStream_t st)
@@ -467,9 +517,10 @@ cudaError_t launch_nusselt(int dim, int prec, const void* f, const void* g, cons
     const long n_face = ax == 0 ? (long)geo.ny * geo.nz : (ax == 1 ? (long)geo.nx * geo.nz
                                                                     : (long)geo.nx * geo.ny);
     const int nb = (int)(nusselt_scratch_doubles(n_face) / 5);
+    const int threads = (int)std::min<long>(256, (n_face + 31) / 32 * 32);
     LBM_DISPATCH(dim, prec, {
         using T = typename S::T;
-        nusselt_kernel<S, D><<<nb, 256, 0, st>>>((const T*)f, (const T*)g, geo, hc.T_ref, face,
+        nusselt_kernel<S, D><<<nb, threads, 0, st>>>((const T*)f, (const T*)g, geo, hc.T_ref, face,
                                                  (int)n_face, scale, profile, scratch, ticket, result);
     });
     return cudaGetLastError();

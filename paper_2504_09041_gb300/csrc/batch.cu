@@ -138,6 +138,8 @@ struct lbm_batch_s {
     void* members = nullptr;
     unsigned* status = nullptr;
     double *nu_profile = nullptr, *nu_scratch = nullptr, *nu_result = nullptr;
+    double nu_host[5] = {};   // result of lbm_batch_nusselt, written by the kernel where host_writes()
+    bool host_writes = false;
     unsigned* ticket = nullptr;
     int n_tiles = 0, tile_x = 64, tile_y = 2, ctas_per_sm = 0, sms = 0;
     cudaStream_t stream = nullptr, capture_stream = nullptr;
@@ -359,6 +361,7 @@ int lbm_batch_create(int lattice, int count, const int* nx, const int* ny, const
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
     if (b->sms < 1) b->sms = 1;
+    b->host_writes = lbm::host_writes();
     const size_t bytes = 9ULL * b->total * elem_bytes(b->prec);
     long max_face = 0;
     for (auto& P : b->plans) max_face = std::max<long>(max_face, std::max(P.nx, P.ny));
@@ -548,9 +551,10 @@ int lbm_batch_nusselt(lbm_batch b, int member, int face, double* mean, double* n
     const size_t o = b->off[member] * elem_bytes(b->prec);
     B_CK(b, lbm::launch_nusselt(2, b->prec, (char*)b->f[b->cur] + o, (char*)b->g[b->cur] + o, P.geo, P.hc,
                                 face, -s * P.L / P.dT, b->nu_profile, b->nu_scratch, b->ticket,
-                                b->nu_result, b->stream));
-    double r[5];
-    B_CK(b, cudaMemcpyAsync(r, b->nu_result, sizeof r, cudaMemcpyDeviceToHost, b->stream));
+                                b->host_writes ? b->nu_host : b->nu_result, b->stream));
+    double* const r = b->nu_host;
+    if (!b->host_writes)
+        B_CK(b, cudaMemcpyAsync(r, b->nu_result, sizeof b->nu_host, cudaMemcpyDeviceToHost, b->stream));
     B_CK(b, cudaStreamSynchronize(b->stream));
     const long n = face < 2 ? P.ny : P.nx;
     if (mean) *mean = r[0] / (double)n;

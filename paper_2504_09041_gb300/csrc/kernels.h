@@ -109,7 +109,11 @@ cudaError_t launch_set_pops(int dim, int prec, void* f, void* g, const Geometry&
 // scratch must hold nusselt_scratch_doubles(n_face) doubles plus one unsigned ticket (ticket
 // must be zero on entry and is left zero on exit).  result receives
 // {sum, max, argmax, min, argmin} as doubles.
+// profile may be any device memory, result too, or host memory where host_writes() holds.
 size_t nusselt_scratch_doubles(long n_face);
+// Kernels of the current device may write ordinary host memory (the CPU's page tables serve the GPU, as
+// on Grace-Blackwell): a few result numbers then need no copy of their own.
+bool host_writes();
 cudaError_t launch_nusselt(int dim, int prec, const void* f, const void* g, const Geometry& geo,
                            const HostCoeffs& hc, int face, double scale, double* profile,
                            double* scratch, unsigned* ticket, double* result, cudaStream_t st);

@@ -430,9 +430,13 @@ __device__ __forceinline__ void store_node_f16s(__half* __restrict__ fout, __hal
                                                 const float* df, const float* dg, int sr)
 {
     unsigned h2[(QF + QG) / 2];
-    if (sr) pack_node_f16s<QF, QG, true, kScaled>(i, df, dg, h2);
-    else pack_node_f16s<QF, QG, false, kScaled>(i, df, dg, h2);
-    store_packed_f16s<QF, QG, Idx>(fout, gout, n, i, h2);
+    if (sr) {
+        pack_node_f16s<QF, QG, true, kScaled>(i, df, dg, h2);
+        store_packed_f16s<QF, QG, Idx>(fout, gout, n, i, h2);
+    } else {
+        pack_node_f16s<QF, QG, false, kScaled>(i, df, dg, h2);
+        store_packed_f16s<QF, QG, Idx>(fout, gout, n, i, h2);
+    }
 }
 
 // 1 / x to about an ulp: the hardware's approximation y and one step of a power series in its residual

@@ -54,3 +54,33 @@ def test_fields_alone_equal_fields_together(lattice, shape, precision):
         torch.cuda.synchronize()
         assert torch.equal(out, together[name]), name
     lat.close()
+
+
+@pytest.mark.parametrize("lattice,shape,face", [("d2q9", (1, 1, 2), 0), ("d2q9", (1, 31, 2), 1), ("d2q9", (1, 33, 5), 0),
+                                                ("d2q9", (1, 128, 3), 0), ("d2q9", (1, 257, 3), 1),
+                                                ("d3q27", (17, 61, 4), 0), ("d3q27", (1, 2050, 2), 1)])
+@pytest.mark.parametrize("nan_at", [None, 0])
+def test_nusselt_numbers_are_those_of_the_profile(lattice, shape, face, nan_at):
+    """Mean, extrema and their first places against the profile, for faces of one thread up to several
+    blocks; a node that is NaN counts for neither extremum and makes the mean NaN.  The mean's sum of
+    n FP64 terms in another order: n 2^-52 of the largest."""
+    nz, ny, nx = shape
+    lat = L.Lattice(lattice, nx, ny, nz, Ra=1e4, precision="fp64")
+    f, g = lat.get_populations()
+    g = synth.perturbed(g, 7, 0.1)
+    if nan_at is not None:
+        g[0, 0, 0, nx - 1 if face else 0] = np.nan     # the rest link of the face's first node
+    lat.set_populations(f, g)
+    prof = lat.nusselt_profile(face).cpu().numpy()
+    mean, mx, mn, jmx, jmn = lat.nusselt(face)
+    lat.close()
+    assert prof.size == ny * nz
+    if nan_at is None:
+        assert mean == pytest.approx(prof.mean(), abs=prof.size * 2.0 ** -52 * np.abs(prof).max())
+    else:
+        assert np.isnan(mean) and np.isnan(prof[0])
+        if prof.size == 1:
+            assert mx == -np.inf and mn == np.inf
+            return
+    assert (mx, mn) == (np.nanmax(prof), np.nanmin(prof))
+    assert (jmx, jmn) == (int(np.nanargmax(prof)), int(np.nanargmin(prof)))
