@@ -162,6 +162,17 @@ __device__ __forceinline__ unsigned sr_pair_bits(unsigned seed)
 template <class S>
 struct has_unit_step : std::integral_constant<bool, !std::is_same<S, StoreF32>::value> {};
 
+// Loads of two neighbouring FP16 values in a kernel that has called wait_previous_step; p on 4 bytes.
+__device__ __forceinline__ unsigned ld_step_pair(const __half* p)
+{
+    unsigned v;
+    asm volatile("ld.global.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ __half low_half(unsigned w) { return __ushort_as_half((unsigned short)(w & 0xffffu)); }
+__device__ __forceinline__ __half high_half(unsigned w) { return __ushort_as_half((unsigned short)(w >> 16)); }
+
 // Box geometry and wall description shared by every kernel.
 struct Geometry {
     int nx, ny, nz;

@@ -20,11 +20,14 @@ namespace lbm {
 template <class R>
 using Coeffs2D = Coeffs<R, 9, 9>;
 
+// Which lattices a pull reads.
+enum { kFlow = 1, kEnergy = 2, kBoth = 3 };
+
 // Streaming (Eqs. LBMsteps-stream, LBMsteps-streamg) with half-way bounce-back for f, and
 // bounce-back (adiabatic) or anti-bounce-back (fixed T) for g at the walls (Sec. 6.1), in
 // deviations: the anti-bounce-back g_a = -g~_abar + 2 w_a T_w becomes
 // gamma_a = -gamma~_abar + 2 w_a (T_w - T_o).
-template <class S, class Idx = size_t, int kPull = kPullDev>
+template <class S, class Idx = size_t, int kPull = kPullDev, int kOf = kBoth>
 __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
                                           const typename S::T* __restrict__ gin, const Geometry& geo,
                                           const NodeWalls<typename S::R>& w, int i, typename S::R T_ref,
@@ -38,15 +41,17 @@ __device__ __forceinline__ void pull_d2q9(const typename S::T* __restrict__ fin,
         R tw;
         const int s = link_source<e9(a, 0), e9(a, 1), 0>(geo, w, i, &out, &dir, &tw);
         const Idx off = out ? (Idx)o * geo.n + i : (Idx)a * geo.n + s;
-        f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
-        const R gv = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
-        g[a] = dir ? anti_bounce<S, kPull>(gv, w9(a), tw, T_ref) : gv;
+        if constexpr ((kOf & kFlow) != 0) f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
+        if constexpr ((kOf & kEnergy) != 0) {
+            const R gv = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
+            g[a] = dir ? anti_bounce<S, kPull>(gv, w9(a), tw, T_ref) : gv;
+        }
     });
 }
 
 // The same pull at a node whose eight neighbours all lie inside the box: no wall and no
 // periodic wrap touches any link, so every population comes straight from its upwind node.
-template <class S, class Idx = size_t, int kPull = kPullDev>
+template <class S, class Idx = size_t, int kPull = kPullDev, int kOf = kBoth>
 __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restrict__ fin,
                                                    const typename S::T* __restrict__ gin,
                                                    const Geometry& geo, int i, typename S::R T_ref,
@@ -56,8 +61,8 @@ __device__ __forceinline__ void pull_d2q9_interior(const typename S::T* __restri
     static_for<9>([&](auto A) {
         constexpr int a = decltype(A)::value;
         const Idx off = (Idx)a * geo.n + (i - (e9(a, 0) + e9(a, 1) * geo.nx));
-        f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
-        g[a] = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
+        if constexpr ((kOf & kFlow) != 0) f[a] = load_link<S, kPull>(fin, off, R(w9(a)));
+        if constexpr ((kOf & kEnergy) != 0) g[a] = load_link<S, kPull>(gin, off, R(w9(a)) * T_ref);
     });
 }
 
@@ -183,17 +188,24 @@ __device__ __forceinline__ void from_central_d2q9(R p[3][3], R f[9], R ux, R uy)
 // deviations e from the rest state moving at u (1, 1/3 on 20 and 02, 1/9 on 22, times kUnits for the
 // flow and T_o for the energy), whose share of the inverse sweeps is the rest weights; so, as in the
 // general form, no O(1) number is rounded on the way to the stored one.
-template <class S, class Idx>
-__device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9], const typename S::R g[9],
-                                                        typename S::T* __restrict__ fout,
-                                                        typename S::T* __restrict__ gout,
-                                                        const Geometry& geo,
-                                                        const UnitCoeffs<typename S::R>& c,
-                                                        unsigned* status, int i)
+template <class R>
+struct FlowSums2D {
+    R drho, jx, jy, Mxx, Myy, Mxy, Mxxy;
+};
+template <class R>
+struct EnergySums2D {
+    R dT, T, jgx, jgy;
+};
+// rho and u of a node, and what both collisions share of the force along y (py = rho u_y).
+template <class R>
+struct Macro2D {
+    R rho, irho, Fy, hF, py, ux, uy;
+};
+
+template <class S>
+__device__ __forceinline__ FlowSums2D<typename S::R> flow_sums_d2q9(const typename S::R f[9])
 {
     using R = typename S::R;
-    constexpr double kS = S::kUnits;
-    const R third = R(1.0 / 3.0), half = R(0.5);
     // raw sums of the flow, rows e_y = -1, 0, 1: (7, 4, 8), (3, 0, 1), (6, 2, 5).  For stored
     // populations the rest weights come off exactly: (a - 2 w) + c has no rounding.
     R k0[3], d[3], s[3];
@@ -212,24 +224,59 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             }
         }
     }
-    const R Myy = k0[0] + k0[2], drho = Myy + k0[1];
-    const R jx = (d[0] + d[2]) + d[1], jy = k0[2] - k0[0];
-    const R Mxx = (s[0] + s[2]) + s[1], Mxy = d[2] - d[0], Mxxy = s[2] - s[0];
-    // raw sums of the energy, over opposite links: g = dT + T0.  Stored populations are summed as they
-    // are (T0 = 0), which also keeps the small ones beside a cold wall exact.
-    const R T0 = S::kFull ? R(0) : R(kS) * c.T_ref;
-    const R dT = (g[0] + ((g[1] + g[3]) + (g[2] + g[4]))) + ((g[5] + g[7]) + (g[6] + g[8]));
+    FlowSums2D<R> m;
+    m.Myy = k0[0] + k0[2];
+    m.drho = m.Myy + k0[1];
+    m.jx = (d[0] + d[2]) + d[1];
+    m.jy = k0[2] - k0[0];
+    m.Mxx = (s[0] + s[2]) + s[1];
+    m.Mxy = d[2] - d[0];
+    m.Mxxy = s[2] - s[0];
+    return m;
+}
+
+// Raw sums of the energy, over opposite links: g = dT + T0.  Stored populations are summed as they are
+// (T0 = 0), which also keeps the small ones beside a cold wall exact.
+template <class S>
+__device__ __forceinline__ EnergySums2D<typename S::R> energy_sums_d2q9(const typename S::R g[9],
+                                                                        const UnitCoeffs<typename S::R>& c)
+{
+    using R = typename S::R;
+    EnergySums2D<R> m;
+    m.dT = (g[0] + ((g[1] + g[3]) + (g[2] + g[4]))) + ((g[5] + g[7]) + (g[6] + g[8]));
     const R d57 = g[5] - g[7], d68 = g[6] - g[8];
-    const R jgx = (g[1] - g[3]) + (d57 - d68), jgy = (g[2] - g[4]) + (d57 + d68);
-    const R T = S::kFull ? dT : T0 + dT, rho = R(kS) + drho;
-    check_node_bits(status, rho, T);
+    m.jgx = (g[1] - g[3]) + (d57 - d68);
+    m.jgy = (g[2] - g[4]) + (d57 + d68);
+    m.T = S::kFull ? m.dT : R(S::kUnits) * c.T_ref + m.dT;
+    return m;
+}
 
-    const R irho = recip(rho);
-    const R Fy = c.gbeta * (S::kFull ? dT - c.T_ref : dT), hF = half * Fy;
-    const R py = jy + hF;                        // rho u_y
-    const R ux = jx * irho, uy = py * irho;
+template <class S>
+__device__ __forceinline__ Macro2D<typename S::R> macro_d2q9(typename S::R drho, typename S::R jx, typename S::R jy,
+                                                             typename S::R dT, const UnitCoeffs<typename S::R>& c)
+{
+    using R = typename S::R;
+    Macro2D<R> m;
+    m.rho = R(S::kUnits) + drho;
+    m.irho = recip(m.rho);
+    m.Fy = c.gbeta * (S::kFull ? dT - c.T_ref : dT);
+    m.hF = R(0.5) * m.Fy;
+    m.py = jy + m.hF;
+    m.ux = jx * m.irho;
+    m.uy = m.py * m.irho;
+    return m;
+}
+
+template <class S>
+__device__ __forceinline__ void collide_flow_d2q9_unit(const FlowSums2D<typename S::R>& m, const Macro2D<typename S::R>& u,
+                                                       const UnitCoeffs<typename S::R>& c, typename S::R df[9])
+{
+    using R = typename S::R;
+    constexpr double kS = S::kUnits;
+    const R third = R(1.0 / 3.0), half = R(0.5);
+    const R drho = m.drho, jx = m.jx, Mxx = m.Mxx, Myy = m.Myy, Mxy = m.Mxy, Mxxy = m.Mxxy;
+    const R rho = u.rho, irho = u.irho, Fy = u.Fy, hF = u.hF, py = u.py, ux = u.ux, uy = u.uy;
     const R uxh = half * ux, uyh = half * uy;
-
     R p[3][3];   // [y link][x moment]: x moments of order 1, 2 halved
     {
         // pre-collision central moments of order 2 (e20, e02: less kS / 3) and kappa_21
@@ -264,11 +311,21 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             unline(e20h, R(kS / 6.0) + e20h, half * h21, R(0.25) * e22, uy, uyh, p[0][2], p[1][2], p[2][2]);
         }
     }
-    R df[9], dg[9];
     unline(p[0][0], R(kS / 6.0) + p[0][0], p[0][1], p[0][2], ux, uxh, df[7], df[4], df[8]);
     unline(p[1][0], R(kS * 2.0 / 3.0) + p[1][0], p[1][1], p[1][2], ux, uxh, df[3], df[0], df[1]);
     unline(p[2][0], R(kS / 6.0) + p[2][0], p[2][1], p[2][2], ux, uxh, df[6], df[2], df[5]);
 
+}
+
+template <class S>
+__device__ __forceinline__ void collide_energy_d2q9_unit(const EnergySums2D<typename S::R>& m, typename S::R ux,
+                                                         typename S::R uy, const UnitCoeffs<typename S::R>& c,
+                                                         typename S::R dg[9])
+{
+    using R = typename S::R;
+    const R half = R(0.5), uxh = half * ux, uyh = half * uy;
+    const R dT = m.dT, T = m.T, jgx = m.jgx, jgy = m.jgy;
+    R p[3][3];
     // energy: T, (1 - omega) eta_1, then c_s^2 T, (2/3) c_s^2 t_1 and c_s^4 T
     {
         const R t10 = c.kg[0] * (jgx - ux * T);
@@ -288,6 +345,7 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
             unline(p[1][0], p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
             unline(p[2][0], p[2][0], p[2][1], p[2][2], ux, uxh, dg[6], dg[2], dg[5]);
         } else {
+            const R T0 = R(S::kUnits) * c.T_ref;
             const R c6 = R(1.0 / 6.0) * T0, c23 = R(2.0 / 3.0) * T0;
             unline(p[0][0], c6 + p[0][0], p[0][1], p[0][2], ux, uxh, dg[7], dg[4], dg[8]);
             unline(p[1][0], c23 + p[1][0], p[1][1], p[1][2], ux, uxh, dg[3], dg[0], dg[1]);
@@ -295,6 +353,24 @@ __device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9]
         }
     }
 
+}
+
+template <class S, class Idx>
+__device__ __forceinline__ void collide_store_d2q9_unit(const typename S::R f[9], const typename S::R g[9],
+                                                        typename S::T* __restrict__ fout,
+                                                        typename S::T* __restrict__ gout,
+                                                        const Geometry& geo,
+                                                        const UnitCoeffs<typename S::R>& c,
+                                                        unsigned* status, int i)
+{
+    using R = typename S::R;
+    const FlowSums2D<R> mf = flow_sums_d2q9<S>(f);
+    const EnergySums2D<R> mg = energy_sums_d2q9<S>(g, c);
+    const Macro2D<R> u = macro_d2q9<S>(mf.drho, mf.jx, mf.jy, mg.dT, c);
+    check_node_bits(status, u.rho, mg.T);
+    R df[9], dg[9];
+    collide_flow_d2q9_unit<S>(mf, u, c, df);
+    collide_energy_d2q9_unit<S>(mg, u.ux, u.uy, c, dg);
     if constexpr (std::is_same<S, StoreF16S>::value) {
         store_node_f16s<9, 9, Idx, true>(fout, gout, (Idx)geo.n, i, df, dg, c.fp16_sr);
     } else {
@@ -364,6 +440,32 @@ __device__ __forceinline__ void collide_store_d2q9(typename S::R f[9], typename 
 template <class S, bool kUnit>
 using StepCoeffs2D = typename std::conditional<kUnit, UnitCoeffs<typename S::R>, Coeffs2D<typename S::R>>::type;
 
+// The pull of one node of the step.
+template <class S, class Idx, int kPull, int kOf, class C>
+__device__ __forceinline__ void pull_by_warp_d2q9(const typename S::T* __restrict__ fin,
+                                                  const typename S::T* __restrict__ gin, const Geometry& geo,
+                                                  const C& c, int x, int y, int i, typename S::R f[9],
+                                                  typename S::R g[9])
+{
+    using R = typename S::R;
+    // Which pull: decided per warp where possible, so that a warp holding an x-wall node of an
+    // interior row runs one x-only pull instead of both the interior and the general pull.
+    const bool y_in = y > 0 && y < geo.ny - 1;
+    const bool in = y_in && x > 0 && x < geo.nx - 1;
+    const unsigned lanes = __activemask();
+    if (__all_sync(lanes, in)) {
+        pull_d2q9_interior<S, Idx, kPull, kOf>(fin, gin, geo, i, c.T_ref, f, g);
+    } else if (__all_sync(lanes, y_in)) {
+        const NodeWalls<R> w = node_walls_x<R>(geo, x, y, 0);
+        pull_d2q9<S, Idx, kPull, kOf>(fin, gin, geo, w, i, c.T_ref, f, g);
+    } else if (in) {
+        pull_d2q9_interior<S, Idx, kPull, kOf>(fin, gin, geo, i, c.T_ref, f, g);
+    } else {
+        const NodeWalls<R> w = node_walls<R>(geo, x, y, 0, 2);
+        pull_d2q9<S, Idx, kPull, kOf>(fin, gin, geo, w, i, c.T_ref, f, g);
+    }
+}
+
 // One time step at one node: pull, macroscopic fields (App. A Step 7, App. B Step 7, Sec. 6.1
 // Boussinesq force), collide f and g, store.  kUnit: the reduced collision above.
 template <class S, class Idx, bool kUnit = false>
@@ -378,29 +480,14 @@ __device__ __forceinline__ void node_step_d2q9(const typename S::T* __restrict__
     constexpr int kPull = kPullAfter | (kUnit ? kPullRaw : kPullDev);
     const int i = x + geo.nx * y;
     R f[9], g[9];
-    // Which pull: decided per warp where possible, so that a warp holding an x-wall node of an
-    // interior row runs one x-only pull instead of both the interior and the general pull.
-    const bool y_in = y > 0 && y < geo.ny - 1;
-    const bool in = y_in && x > 0 && x < geo.nx - 1;
-    const unsigned lanes = __activemask();
-    if (__all_sync(lanes, in)) {
-        pull_d2q9_interior<S, Idx, kPull>(fin, gin, geo, i, c.T_ref, f, g);
-    } else if (__all_sync(lanes, y_in)) {
-        const NodeWalls<R> w = node_walls_x<R>(geo, x, y, 0);
-        pull_d2q9<S, Idx, kPull>(fin, gin, geo, w, i, c.T_ref, f, g);
-    } else if (in) {
-        pull_d2q9_interior<S, Idx, kPull>(fin, gin, geo, i, c.T_ref, f, g);
-    } else {
-        const NodeWalls<R> w = node_walls<R>(geo, x, y, 0, 2);
-        pull_d2q9<S, Idx, kPull>(fin, gin, geo, w, i, c.T_ref, f, g);
-    }
-
+    pull_by_warp_d2q9<S, Idx, kPull, kBoth>(fin, gin, geo, c, x, y, i, f, g);
     if constexpr (kUnit) {
         collide_store_d2q9_unit<S, Idx>(f, g, fout, gout, geo, c, status, i);
     } else {
         collide_store_d2q9<S, Idx>(f, g, fout, gout, geo, c, status, i);
     }
 }
+
 template <class S, class Idx, bool kUnit = false>
 __global__ void __launch_bounds__(256)
     step_d2q9_kernel(const typename S::T* __restrict__ fin, const typename S::T* __restrict__ gin,
@@ -412,6 +499,162 @@ __global__ void __launch_bounds__(256)
     wait_previous_step();
     if (x >= geo.nx || y >= geo.ny) return;
     node_step_d2q9<S, Idx, kUnit>(fin, gin, fout, gout, geo, c, status, x, y);
+}
+
+// FP16 storage, reduced collision, two x-adjacent nodes per thread (x even); see
+// step_d3q27_pair_f16s_kernel.  A node takes 15 loads and 9 stores instead of 18 and 18.
+// 4096 x 2048: 105 us per step against 133; 1024 x 512, in L2, 7.9 against 8.5; 512^2 is even, and smaller
+// boxes lose warps.  Bitwise the results of the one-node kernel.
+__device__ __forceinline__ void pair_node_d2q9(const float f[9], const float g[9], const UnitCoeffs<float>& c,
+                                               unsigned* status, int i, unsigned h2[9])
+{
+    using S = StoreF16S;
+    const FlowSums2D<float> mf = flow_sums_d2q9<S>(f);
+    const EnergySums2D<float> mg = energy_sums_d2q9<S>(g, c);
+    const Macro2D<float> u = macro_d2q9<S>(mf.drho, mf.jx, mf.jy, mg.dT, c);
+    check_node_bits(status, u.rho, mg.T);
+    float df[9], dg[9];
+    collide_flow_d2q9_unit<S>(mf, u, c, df);
+    collide_energy_d2q9_unit<S>(mg, u.ux, u.uy, c, dg);
+    if (c.fp16_sr) pack_node_f16s<9, 9, true, true>(i, df, dg, h2);
+    else pack_node_f16s<9, 9, false, true>(i, df, dg, h2);
+}
+
+// The values of a node on an x wall (or x wrap) of an interior row that arrive through x.
+__device__ __forceinline__ void fix_x_edge_d2q9_f16s(const __half* __restrict__ fin, const __half* __restrict__ gin,
+                                                     const Geometry& geo, int x, int y, int i, float T_ref, float f[9],
+                                                     float g[9])
+{
+    using S = StoreF16S;
+    const NodeWalls<float> w = node_walls_x<float>(geo, x, y, 0);
+    static_for<9>([&](auto A) {
+        constexpr int a = decltype(A)::value;
+        constexpr int ex = e9(a, 0), o = opp9(a);
+        if constexpr (ex != 0) {
+            if (ex == 1 ? x == 0 : x == geo.nx - 1) {
+                bool out, dir;
+                float tw;
+                const int s = link_source<ex, e9(a, 1), 0>(geo, w, i, &out, &dir, &tw);
+                const unsigned off = out ? (unsigned)o * geo.n + i : (unsigned)a * geo.n + s;
+                f[a] = S::raw(ld_step(fin + off));
+                const float gv = S::raw(ld_step(gin + off));
+                g[a] = dir ? anti_bounce<S, kPullRaw>(gv, w9(a), tw, T_ref) : gv;
+            }
+        }
+    });
+}
+
+template <class Idx>
+__global__ void __launch_bounds__(256)
+    step_d2q9_pair_f16s_kernel(const __half* __restrict__ fin, const __half* __restrict__ gin, __half* __restrict__ fout,
+                               __half* __restrict__ gout, Geometry geo, UnitCoeffs<float> c, unsigned* status, bool flip)
+{
+    using S = StoreF16S;
+    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = (flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
+    wait_previous_step();
+    if (x >= geo.nx || y >= geo.ny) return;
+    const int i = x + geo.nx * y;
+    const Idx n = (Idx)geo.n;
+    unsigned out0[9], out1[9];
+    float f[9], g[9];
+    if (y > 0 && y < geo.ny - 1) {
+        unsigned w[18];
+        // an x link that would leave the row reads its partner's place instead and is replaced below: the
+        // row behind the last one may end the buffer
+        const int lo = x > 0 ? i - 1 : i, hi = x + 2 < geo.nx ? i + 2 : i + 1;
+        static_for<18>([&](auto A) {
+            constexpr int k = decltype(A)::value, a = k % 9, ex = e9(a, 0);
+            const __half* p = (k < 9 ? fin : gin) + (Idx)a * n;
+            const int row = e9(a, 1) * geo.nx;
+            if constexpr (ex == 0) {
+                w[k] = ld_step_pair(p + (i - row));
+            } else {
+                const int s0 = (ex == 1 ? lo : i + 1) - row, s1 = (ex == 1 ? i : hi) - row;
+                w[k] = (unsigned)__half_as_ushort(ld_step(p + s0)) | (unsigned)__half_as_ushort(ld_step(p + s1)) << 16;
+            }
+        });
+        static_for<9>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            f[a] = S::raw(low_half(w[a]));
+            g[a] = S::raw(low_half(w[9 + a]));
+        });
+        if (x == 0) fix_x_edge_d2q9_f16s(fin, gin, geo, x, y, i, c.T_ref, f, g);
+        pair_node_d2q9(f, g, c, status, i, out0);
+        static_for<9>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            f[a] = S::raw(high_half(w[a]));
+            g[a] = S::raw(high_half(w[9 + a]));
+        });
+        if (x + 2 == geo.nx) fix_x_edge_d2q9_f16s(fin, gin, geo, x + 1, y, i + 1, c.T_ref, f, g);
+    } else {
+        constexpr int kPull = kPullAfter | kPullRaw;
+        pull_d2q9<S, Idx, kPull>(fin, gin, geo, node_walls<float>(geo, x, y, 0, 2), i, c.T_ref, f, g);
+        pair_node_d2q9(f, g, c, status, i, out0);
+        pull_d2q9<S, Idx, kPull>(fin, gin, geo, node_walls<float>(geo, x + 1, y, 0, 2), i + 1, c.T_ref, f, g);
+    }
+    pair_node_d2q9(f, g, c, status, i + 1, out1);
+    static_for<18>([&](auto A) {
+        constexpr int a = decltype(A)::value;
+        const unsigned v = __byte_perm(out0[a / 2], out1[a / 2], (a & 1) ? 0x7632 : 0x5410);
+        __half* p = (a < 9 ? fout : gout) + (Idx)(a % 9) * n;
+        *reinterpret_cast<unsigned*>(p + i) = v;
+    });
+}
+
+// FP64, reduced collision, small boxes: the two lattices of 32 nodes on two warps of a block, which swap
+// their sums (T, and rho and j) once.  A sub-partition takes an FP64 instruction per 64 cycles however
+// few lanes or warps it has, so while warps are fewer than the 608 sub-partitions the step lasts as
+// long as one warp's FP64 instructions: about 105 here (the flow's) against 175.  64^2: 5.4 us per step
+// against 7.6, 96^2 6.0 against 7.6; with more warps than sub-partitions the second macro_d2q9 only
+// costs (128^2 8.7 against 8.3).
+// Each warp's arithmetic is that of the one-warp kernel; the states are bitwise the same.
+template <class Idx>
+__global__ void __launch_bounds__(64)
+    step_d2q9_split_f64_kernel(const double* __restrict__ fin, const double* __restrict__ gin, double* __restrict__ fout,
+                               double* __restrict__ gout, Geometry geo, UnitCoeffs<double> c, unsigned* status)
+{
+    using S = StoreF64;
+    __shared__ double swap[4][32];
+    const int lane = threadIdx.x & 31;
+    const bool flow = threadIdx.x < 32;
+    const int x = blockIdx.x * 32 + lane, y = blockIdx.y;
+    const int i = x + geo.nx * y;
+    const bool active = x < geo.nx;
+    wait_previous_step();
+    double v[9], out[9];
+    FlowSums2D<double> mf{};
+    EnergySums2D<double> mg{};
+    if (active) {
+        if (flow) {
+            pull_by_warp_d2q9<S, Idx, kPullAfter | kPullRaw, kFlow>(fin, gin, geo, c, x, y, i, v, v);
+            mf = flow_sums_d2q9<S>(v);
+            swap[0][lane] = mf.drho;
+            swap[1][lane] = mf.jx;
+            swap[2][lane] = mf.jy;
+        } else {
+            pull_by_warp_d2q9<S, Idx, kPullAfter | kPullRaw, kEnergy>(fin, gin, geo, c, x, y, i, v, v);
+            mg = energy_sums_d2q9<S>(v, c);
+            swap[3][lane] = mg.dT;
+        }
+    }
+    __syncthreads();
+    if (!active) return;
+    const Macro2D<double> u = macro_d2q9<S>(swap[0][lane], swap[1][lane], swap[2][lane], swap[3][lane], c);
+    if (flow) {
+        collide_flow_d2q9_unit<S>(mf, u, c, out);
+        static_for<9>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            S::store_dev(fout, (Idx)a * geo.n + i, out[a], w9(a));
+        });
+    } else {
+        check_node_bits(status, u.rho, mg.T);
+        collide_energy_d2q9_unit<S>(mg, u.ux, u.uy, c, out);
+        static_for<9>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            gout[(Idx)a * geo.n + i] = out[a];
+        });
+    }
 }
 
 }  // namespace lbm

@@ -1022,9 +1022,6 @@ __global__ void __maxnreg__(LBM_MAXREG3D)
 #define LBM_MAXREG3D_PAIR 96
 #endif
 
-__device__ __forceinline__ __half low_half(unsigned w) { return __ushort_as_half((unsigned short)(w & 0xffffu)); }
-__device__ __forceinline__ __half high_half(unsigned w) { return __ushort_as_half((unsigned short)(w >> 16)); }
-
 // Both collisions of one node of a pair, rounded to packed storage.
 __device__ __forceinline__ void pair_node(const float f[27], const float g[15], const UnitCoeffs<float>& c,
                                           unsigned* status, int i, unsigned h2[21])

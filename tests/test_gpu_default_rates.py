@@ -108,3 +108,46 @@ def test_fp16s_node_pairs_equal_single_nodes(kind, shape, stochastic):
         states.append(gpu.get_state()[64:])
         gpu.close()
     assert np.array_equal(states[0], states[1])
+
+
+@pytest.mark.parametrize("kind,shape", [("cavity", (1, 64, 64)), ("rb", (1, 33, 70)), ("periodic", (1, 5, 31)),
+                                        ("cavity", (1, 3, 2)), ("rb", (1, 1, 5)), ("cavity", (1, 149, 96)),
+                                        ("rb", (1, 448, 32)), ("rb", (1, 449, 32))])
+def test_fp64_split_step_equals_the_one_warp_step(kind, shape):
+    """Small FP64 boxes run the two lattices of a node on two warps; a chosen block_x selects the
+    one-warp kernel.  Bitwise equal up to and just above the size where the rule changes over."""
+    nz, ny, nx = shape
+    states = []
+    for block in (0, 32):
+        gpu = L.Lattice("d2q9", nx, ny, Ra=1e4, walls=walls_pair(kind, 2)[0], precision="fp64")
+        gpu.set_param("gbeta", 3e-3)
+        if block:
+            gpu.set_param("block_x", block)
+        f, g = gpu.get_populations()
+        gpu.set_populations(synth.perturbed(f, 3, 0.05), synth.perturbed(g, 4, 0.05))
+        gpu.step(40)
+        gpu.sync()
+        states.append(gpu.get_state()[64:])
+        gpu.close()
+    assert np.array_equal(states[0], states[1])
+
+
+@pytest.mark.parametrize("kind,shape,stochastic", [("cavity", (1, 601, 500), 1), ("rb", (1, 512, 1024), 0),
+                                                   ("periodic", (1, 131070, 4), 1), ("rb", (1, 3, 131074), 1)])
+def test_fp16s_node_pairs_equal_single_nodes_2d(kind, shape, stochastic):
+    """Boxes of 300,000 nodes and more with an even nx update two nodes per thread; a chosen block_x
+    selects the one-node kernel.  Bitwise equal; an odd number of steps, so that both walking
+    directions run."""
+    nz, ny, nx = shape
+    states = []
+    for block in (0, 64):
+        gpu = L.Lattice("d2q9", nx, ny, Ra=1e4, walls=walls_pair(kind, 2, seed=5, perturb=0.05)[0], precision="fp16s")
+        gpu.set_param("fp16_stochastic", stochastic)
+        gpu.set_param("gbeta", 3e-3)
+        if block:
+            gpu.set_param("block_x", block)
+        gpu.step(5)
+        gpu.sync()
+        states.append(gpu.get_state()[64:])
+        gpu.close()
+    assert np.array_equal(states[0], states[1])
