@@ -139,7 +139,7 @@ LBM_API int lbm_set_omegas(lbm_handle h, const double* om_f, int n_f, const doub
  * smaller than half an FP16 step accumulate in expectation; 0 rounds to nearest), "adjoint_arith" (arithmetic of lbm_adjoint_step's vector-Jacobian products and adjoint state: 2, the default, double-float, i.e. pairs of FP32
  * numbers with a 48-bit significand evaluated on the FP32 pipes; 1 FP64; 0 FP32), "adjoint_fp64" (0 or 1: the same as "adjoint_arith" 0 or 1),
  * "adjoint_sync" (thread blocks of the adjoint kernel: 0 = 64 x 2; 1-4 = 64 x 4, 128 x 2 (the
- * default), 32 x 4, 64 x 2 whose warps pass a barrier between the phases of the node's work so
+ * default; 32 x 2 beyond one wave of them), 32 x 4, 64 x 2 whose warps pass a barrier between the phases of the node's work so
  * that they share the instruction fetches of the long unrolled product; results agree to
  * rounding), "adjoint_overlap" (1, the default: lbm_adjoint_step recomputes the next segment's
  * states on a second, low-priority stream while the adjoint steps of the current one run, with

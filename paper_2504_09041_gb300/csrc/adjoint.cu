@@ -26,9 +26,14 @@ static cudaError_t run_adjoint(const void* f_prev, const void* g_prev, const voi
     using T = typename S::T;
     using R = typename S::R;
     if (hc.adj_sync) {
-        // thread blocks of the barrier-phased kernel: 64x4, 128x2, 32x4 or 64x2
-        const int shapes[5][2] = {{0, 0}, {64, 4}, {128, 2}, {32, 4}, {64, 2}};
-        const dim3 b(shapes[hc.adj_sync][0], shapes[hc.adj_sync][1], 1);
+        // thread blocks of the barrier-phased kernel: 64x4, 128x2, 32x4 or 64x2.  The default, 128x2, fits
+        // two blocks on an SM; a box of more than one wave of them takes 32x2, eight to an SM, whose
+        // last wave is finer (320^2: 23.0 us per adjoint step, forward passes included, against 25.8;
+        // within one wave 128x2 is the faster by 1-2 %, 256^2 15.8 against 16.0)
+        const int shapes[6][2] = {{0, 0}, {64, 4}, {128, 2}, {32, 4}, {64, 2}, {32, 2}};
+        const bool over = hc.adj_sync == 2 && (long)((geo.nx + 127) / 128) * ((geo.ny + 1) / 2) > 2 * 152;
+        const int* shape = shapes[over ? 5 : hc.adj_sync];
+        const dim3 b(shape[0], shape[1], 1);
         const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
         auto kern = unit_rates_2d(hc) ? adjoint_step_d2q9_kernel<S, RT, true, true> : adjoint_step_d2q9_kernel<S, RT, true>;
         return launch_step_kernel(kern, grid, b, st, (const T*)f_prev, (const T*)g_prev, (const RT*)mu_in, (RT*)mu_out,

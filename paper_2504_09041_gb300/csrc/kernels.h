@@ -36,8 +36,8 @@ struct HostCoeffs {
     int fp16_sr;   // F16S storage: stochastic (1) or nearest (0) rounding of stored deviations
     int index64;   // 1: the step uses 64-bit element offsets even where 32-bit ones suffice
     int rows3d;    // 3D FP32 / FP16S step: rows of its column each thread updates (1, 2 or 4; 0 automatic)
-    int adj_sync;  // adjoint step blocks: 0 = 64x2; with phase barriers 1 = 64x4, 2 = 128x2 (default),
-                   // 3 = 32x4, 4 = 64x2
+    int adj_sync;  // adjoint step blocks: 0 = 64x2; with phase barriers 1 = 64x4, 2 = 128x2 (default;
+                   // 32x2 in large boxes), 3 = 32x4, 4 = 64x2
 };
 
 size_t storage_bytes(int prec);
