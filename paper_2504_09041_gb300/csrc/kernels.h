@@ -200,13 +200,14 @@ inline auto make_step_coeffs(const HostCoeffs& h)
 //   threads (256^3 FP32: 16.4 against 15.8 GLUPS); 32 x 1 where a row ends in a half-empty block
 //   (131 x 93 x 77: FP32 64.0 us against 68.7, FP16S 45.3 against 51.7, FP64 1273 against 1288);
 //   128 x 1 from two million nodes on, where rows fill such blocks (256^3: FP32 849 us against 853,
-//   FP16S 826 against 832; but 64^3 15.8 against 14.5).
+//   FP16S 826 against 832; but 64^3 15.8 against 14.5).  Above 65535 rows two rows of them, as in 2D.
 inline dim3 block_shape(const Geometry& g, int prec, int dim, dim3 chosen = dim3(0, 0, 0))
 {
     if (chosen.x > 0) return dim3(chosen.x, chosen.y, 1);
     const int warps = (g.nx + 31) / 32;   // per row
-    if (dim == 3) return dim3(warps & 1 ? 32 : (warps & 3 || g.n < (1 << 21) ? 64 : 128), 1, 1);
-    if (prec == kF64) return dim3(32, g.ny > 65535 ? 2 : 1, 1);
+    const int rows = g.ny > 65535 ? 2 : 1;
+    if (dim == 3) return dim3(warps & 1 ? 32 : (warps & 3 || g.n < (1 << 21) ? 64 : 128), rows, 1);
+    if (prec == kF64) return dim3(32, rows, 1);
     return g.nx > 32 ? dim3(64, 2, 1) : dim3(32, 4, 1);
 }
 

@@ -151,3 +151,30 @@ def test_fp16s_node_pairs_equal_single_nodes_2d(kind, shape, stochastic):
         states.append(gpu.get_state()[64:])
         gpu.close()
     assert np.array_equal(states[0], states[1])
+
+
+@pytest.mark.parametrize("precision,shape", [("fp64", (2, 65537, 3)), ("fp32", (2, 65537, 3)), ("fp16s", (2, 65537, 3)),
+                                             ("fp32", (1, 131070, 4)), ("fp16s", (24, 65537, 4))])
+def test_3d_boxes_taller_than_the_launch_grid(precision, shape):
+    """More than 65535 rows: the default blocks hold two.  Populations equal those of chosen 32 x 8
+    blocks bit by bit.  The read-out covers every row too: the collision conserves the temperature, so
+    the field is the sum of the energy populations after one more step (FP64 to 1e-13; FP32 to 1e-5, 15
+    populations' rounding)."""
+    nz, ny, nx = shape
+    states = []
+    for block in (0, 8):
+        gpu = L.Lattice("d3q27", nx, ny, nz, Ra=1e4, walls=walls_pair("mixed3d", 3, seed=5, perturb=0.05)[0],
+                        precision=precision)
+        if block:
+            gpu.set_param("block_x", 32)
+            gpu.set_param("block_y", block)
+        gpu.step(3)
+        gpu.sync()
+        states.append(gpu.get_state()[64:])
+        if not block and precision != "fp16s":
+            T = gpu.fields()["T"].cpu().numpy()
+            gpu.step(1)
+            _, g = gpu.get_populations()
+            np.testing.assert_allclose(g.sum(axis=0), T, rtol=0, atol=1e-13 if precision == "fp64" else 1e-5)
+        gpu.close()
+    assert np.array_equal(states[0], states[1])
