@@ -692,16 +692,31 @@ int lbm_nusselt(lbm_handle h, int face, double* mean, double* nu_max, double* nu
     return LBM_OK;
 }
 
+// A kernel may write doubles to p itself: device memory, on 8 bytes.  Anything else goes through a copy,
+// which takes any address and reports a bad one.
+static bool kernel_writes_doubles(const void* p)
+{
+    cudaPointerAttributes a{};
+    if (((uintptr_t)p & 7) != 0) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
 int lbm_nusselt_profile(lbm_handle h, int face, double* nu, long n, int device_ptrs)
 {
     if (!h || !nu) return fail(h, LBM_EINVAL, "handle or output is NULL");
     // the face is checked before its length is, and the length before the kernel writes n values
     const bool fits = face >= 0 && face < 2 * h->dim && n == face_nodes(h, face);
-    int rc = nusselt_common(h, face, device_ptrs && fits ? nu : h->nu_profile, h->nu_result);
+    const bool direct = device_ptrs && fits && kernel_writes_doubles(nu);
+    int rc = nusselt_common(h, face, direct ? nu : h->nu_profile, h->nu_result);
     if (rc) return rc;
     if (!fits) return fail(h, LBM_EINVAL, "face %d has %ld nodes, not %ld", face, face_nodes(h, face), n);
-    if (!device_ptrs)
-        LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    if (!direct)
+        LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double),
+                                  device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
     LBM_CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }

@@ -84,3 +84,16 @@ def test_nusselt_numbers_are_those_of_the_profile(lattice, shape, face, nan_at):
             return
     assert (mx, mn) == (np.nanmax(prof), np.nanmin(prof))
     assert (jmx, jmn) == (int(np.nanargmax(prof)), int(np.nanargmin(prof)))
+
+
+def test_wall_profile_into_unaligned_device_memory():
+    """The profile's destination may start at any byte of device memory."""
+    lat = L.Lattice("d2q9", 24, 37, Ra=1e4, precision="fp32")
+    lat.step(3)
+    want = lat.nusselt_profile(0)
+    buf = torch.zeros(8 * 37 + 8, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    L.lbm_nusselt_profile(lat.h, 0, buf.data_ptr() + 4, 37, 1)
+    got = np.frombuffer(buf.cpu().numpy()[4:4 + 8 * 37].tobytes(), dtype=np.float64)
+    lat.close()
+    np.testing.assert_array_equal(got, torch.as_tensor(want).cpu().numpy().reshape(-1))
