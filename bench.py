@@ -413,10 +413,10 @@ def compact_nu_accuracy(nu_acc):
 
 
 # FP64 lane operations per node update of the FP64 steps at the default rates (ncu instruction
-# counts of the FP64 kernels, committed with the profiles; the 3D count is that of the reduced
-# collisions the default rates select) and GB300's FP64 pipe rate: 2 lane operations per SM per
+# counts of the FP64 kernels, committed with the profiles; both counts are those of the
+# reduced collisions the default rates select) and GB300's FP64 pipe rate: 2 lane operations per SM per
 # clock.
-FP64_OPS_PER_NODE = {"d3q27": 866.8, "d2q9": 340.6}
+FP64_OPS_PER_NODE = {"d3q27": 575.4, "d2q9": 176.7}
 FP64_LANE_OPS_PER_SM_CLK = 2
 
 
