@@ -416,7 +416,7 @@ def compact_nu_accuracy(nu_acc):
 # counts of the FP64 kernels, committed with the profiles; both counts are those of the
 # reduced collisions the default rates select) and GB300's FP64 pipe rate: 2 lane operations per SM per
 # clock.
-FP64_OPS_PER_NODE = {"d3q27": 575.4, "d2q9": 176.7}
+FP64_OPS_PER_NODE = {"d3q27": 606.4, "d2q9": 176.7}
 FP64_LANE_OPS_PER_SM_CLK = 2
 
 

@@ -176,6 +176,13 @@ inline UnitCoeffs<R> make_unit_coeffs(const HostCoeffs& h)
     for (int b = 1; b < 4; ++b) c.kg[b - 1] = R(1.0 - h.om_g[b]);
     c.gbeta = R(h.gbeta);
     c.T_ref = R(h.T_ref);
+    c.rest_T = c.T_ref;
+    if constexpr (DIM == 3 && std::is_same<R, double>::value) {
+        const int first[3] = {0, 1, 7};
+        for (int k = 0; k < 3; ++k) c.rest_g[k] = w15(first[k]) * h.T_ref;
+        // (a sum of 53-bit numbers within a factor of 64 of each other: exact in 64 bits and more)
+        c.rest_T = (double)((long double)c.rest_g[0] + 6.0L * c.rest_g[1] + 8.0L * c.rest_g[2]);
+    }
     c.fp16_sr = h.fp16_sr;
     return c;
 }

@@ -85,7 +85,9 @@ __device__ __forceinline__ __half ld_step(const __half* p)
 // The reduced steps (default rates and gravity axis; FP64 and F16S) take the stored number itself (raw) and
 // work in its units: every relation of the step is homogeneous of degree one in the populations, so
 // multiplying them all by kUnits only multiplies the rest state's constants.  kFull: the stored
-// number is the population, not its deviation; the rest state is then taken off in the raw sums.
+// number is the population, not its deviation; the rest state is then taken off in the raw sums (of the
+// flow and, in 3D, of the energy; in 2D the energy is summed and written as stored, see
+// energy_sums_d2q9).
 struct StoreF64 {
     using T = double;
     using R = double;
@@ -202,6 +204,8 @@ struct UnitCoeffs {
     R kf[6];             // 1 - omega of flow slots 4 .. 9
     R kg[3];             // 1 - omega of energy slots 1 .. 3
     R gbeta, T_ref;
+    R rest_g[3];         // 3D, FP64 storage: rest values w_b T_ref of energy links 0, 1-6 and 7-14 ...
+    R rest_T;            // ... and their sum over the 15 links (T_ref in the other forms)
     int fp16_sr;         // as in Coeffs
 };
 

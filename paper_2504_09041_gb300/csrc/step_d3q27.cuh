@@ -613,11 +613,11 @@ __device__ __forceinline__ void raw01_g_d3q15(const R g[15], R& r000, R& r100, R
 // relax with a rate of their own (rho, j and order 2) or that the force multiplies (orders 0-1 in z, up
 // to 2 in x and y); t_210 and t_120 vanish.  The relaxed moments are held as deviations e from the
 // rest state moving at u (1, 1/3, 1/9, 1/27 on the moments even in every direction, times kUnits) and
-// halved once per axis of non-zero order, as the inverse sweeps want them.  About 595 FP64 instructions
-// per node against 867 with the two reduced collisions above alone: 128^3 in FP64 2.33 ms against
-// 3.36 per step; FP16 storage issues 1,012 instructions against 1,249: 81 us against 95 at 128^3, where
+// halved once per axis of non-zero order, as the inverse sweeps want them.  606 FP64 instructions
+// per node against 867 with the two reduced collisions above alone: 128^3 in FP64 2.40 ms against
+// 3.36 per step; FP16 storage issues 1,012 instructions against 1,249: 79 us against 95 at 128^3, where
 // half of it comes from L2.
-// df, dg: the post-collision deviations (FP64 energy: the populations), in storage units.
+// df, dg: the post-collision deviations, in storage units.
 template <class S>
 __device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], const typename S::R g[15],
                                                    const UnitCoeffs<typename S::R>& c, unsigned* status,
@@ -666,10 +666,19 @@ __device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], co
     const R M002 = m[0][0][0] + m[2][0][0];
     const R drho = z0[0][0], jx = z0[0][1], jy = z0[1][0], jz = z1[0][0];
 
-    // energy: T and the first-order moments
-    const R T0 = S::kFull ? R(0) : R(kS) * c.T_ref;   // g = dT + T0, as in 2D
-    const R dT = (g[0] + ((g[1] + g[2]) + ((g[3] + g[4]) + (g[5] + g[6]))))
-               + (((g[7] + g[14]) + (g[8] + g[13])) + ((g[9] + g[12]) + (g[10] + g[11])));
+    // energy: T and the first-order moments.  g = dT + T0: stored populations lose their rest values here,
+    // once per pair of opposite links ((a - 2 w T0) + b has no rounding near the rest state), and gain
+    // them again in the store, so everything between is of the size of the deviations.  Against
+    // 128 bits, T in [0, 1] about 0.5, an update's rounding is 6.5e-18 rms on a population and 2.7e-17 on
+    // their sum, which the collision conserves; summed and written as stored (the better form in 2D) it
+    // is 1.55e-17 and 5.9e-17, and with every link's deviation taken and the moments full, as in
+    // collide_g_d3q15_unit, 1.17e-17 and 3.6e-17.
+    const R T0 = S::kFull ? c.rest_T : R(kS) * c.T_ref;
+    auto pair = [&](int a, int b, R rest) { return S::kFull ? (g[a] - two * rest) + g[b] : g[a] + g[b]; };
+    const R w1 = c.rest_g[1], w7 = c.rest_g[2];
+    const R dT = (((S::kFull ? g[0] - c.rest_g[0] : g[0])
+                   + ((pair(7, 14, w7) + pair(8, 13, w7)) + (pair(9, 12, w7) + pair(10, 11, w7))))
+                  + (pair(1, 2, w1) + pair(3, 4, w1))) + pair(5, 6, w1);
     R gx, gy, gz;
     {   // along the diagonals (+++), (-++), (+-+), (++-)
         const R d1 = g[7] - g[14], d2 = g[8] - g[13], d3 = g[9] - g[12], d4 = g[11] - g[10];
@@ -678,10 +687,10 @@ __device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], co
         gy = (g[3] - g[4]) + (a - b);
         gz = (g[5] - g[6]) + ((d1 - d4) + (d2 + d3));
     }
-    const R T = S::kFull ? dT : T0 + dT, rho = R(kS) + drho;
+    const R T = T0 + dT, rho = R(kS) + drho;
     check_node_bits(status, rho, T);
     const R irho = recip(rho);
-    const R Fz = c.gbeta * (S::kFull ? dT - c.T_ref : dT), hF = half * Fz;
+    const R Fz = c.gbeta * dT, hF = half * Fz;
     const R pz = jz + hF;                                  // rho u_z (u_x, u_y: no force)
     const R ux = jx * irho, uy = jy * irho, uz = pz * irho;
     const R uxh = half * ux, uyh = half * uy, uzh = half * uz;
@@ -765,7 +774,7 @@ __device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], co
         });
     });
 
-    // energy: the moments of collide_g_d3q15_unit as deviations from w T_o
+    // energy: the moments of collide_g_d3q15_unit as deviations from w T0
     {
         constexpr double c3 = 2.0 / 9.0;
         const R rest2 = third * T0;
@@ -775,15 +784,15 @@ __device__ __forceinline__ void collide_d3q27_unit(const typename S::R f[27], co
         const R q110 = ux * t010 + uy * q100, q101 = xt + uz * q100, q011 = uy * t001 + uz * q010;
         const R t2 = third * dT;
         const R q200 = t2 + ux * (t100 + q100), q020 = t2 + uy * (t010 + q010), q002 = t2 + uz * (t001 + q001);
-        const R q020f = S::kFull ? q020 : q020 + rest2;
+        const R q020f = q020 + rest2;
         const R q120 = t100 * (R(c3) + uy * uy) + ux * q020f;
-        const R q012 = t010 * (R(c3) + uz * uz) + uy * (S::kFull ? q002 : q002 + rest2);
-        const R q201 = t001 * (R(c3) + ux * ux) + uz * (S::kFull ? q200 : q200 + rest2);
+        const R q012 = t010 * (R(c3) + uz * uz) + uy * (q002 + rest2);
+        const R q201 = t001 * (R(c3) + ux * ux) + uz * (q200 + rest2);
         const R q111 = uy * xt + uz * q110;
         const R Z1 = q012 - ux * (two * q110 - ux * q010);
-        const R Z2 = R(1.0 / 9.0) * dT + uy * (two * Z1 - uy * (S::kFull ? t2 : third * T));
+        const R Z2 = R(1.0 / 9.0) * dT + uy * (two * Z1 - uy * (third * T));
         const R q220 = Z2 + ux * (two * q120 - ux * q020f);
-        dg[0] = (dT - q200) - (q020 + q002) + two * q220;
+        dg[0] = ((dT - q200) - q020) - q002 + two * q220;
         const R h220 = half * q220, h120 = half * q120, h012 = half * q012, h201 = half * q201;
         const R Sx = half * q200 - h220, Sy = half * q020 - h220, Sz = half * q002 - h220;
         const R Dx = half * q100 - h120, Dy = half * q010 - h012, Dz = half * q001 - h201;
@@ -832,7 +841,7 @@ __device__ __forceinline__ void collide_store_d3q27_unit(const typename S::R f[2
         });
         static_for<15>([&](auto B) {
             constexpr int b = decltype(B)::value;
-            gout[(Idx)b * geo.n + i] = dg[b];
+            S::store_dev(gout, (Idx)b * geo.n + i, dg[b], c.rest_g[b == 0 ? 0 : (b < 7 ? 1 : 2)]);
         });
     }
 }
