@@ -660,7 +660,7 @@ int lbm_fields(lbm_handle h, double* rho, double* ux, double* uy, double* uz, do
     return LBM_OK;
 }
 
-static int nusselt_common(lbm_s* h, int face, double* profile, double* result)
+static int nusselt_common(lbm_s* h, int face, double* result)
 {
     if (face < 0 || face >= 2 * h->dim) return fail(h, LBM_EINVAL, "face %d is not a face of this box", face);
     if (h->geo.kind[face] != LBM_WALL_FIXED_T) return fail(h, LBM_EINVAL, "face %d is not a fixed-temperature wall", face);
@@ -668,8 +668,8 @@ static int nusselt_common(lbm_s* h, int face, double* profile, double* result)
     if (ext[face / 2] < 2) return fail(h, LBM_EINVAL, "fewer than two node layers normal to face %d", face);
     const double s = h->geo.T_wall[face] >= h->hc.T_ref ? 1.0 : -1.0;
     LBM_CK(h, lbm::launch_nusselt(h->dim, h->prec, h->f[h->cur], h->g[h->cur], h->geo, h->hc, face,
-                                  -s * h->L / h->dT, profile, h->nu_scratch, h->ticket, result,
-                                  h->stream));
+                                  -s * h->L / h->dT, h->nu_profile, h->nu_scratch, h->ticket,
+                                  result, h->stream));
     return LBM_OK;
 }
 
@@ -678,7 +678,7 @@ int lbm_nusselt(lbm_handle h, int face, double* mean, double* nu_max, double* nu
 {
     if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
     double* const r = h->nu_host;
-    int rc = nusselt_common(h, face, h->nu_profile, h->host_writes ? r : h->nu_result);
+    int rc = nusselt_common(h, face, h->host_writes ? r : h->nu_result);
     if (rc) return rc;
     if (!h->host_writes)
         LBM_CK(h, cudaMemcpyAsync(r, h->nu_result, sizeof h->nu_host, cudaMemcpyDeviceToHost, h->stream));
@@ -692,31 +692,14 @@ int lbm_nusselt(lbm_handle h, int face, double* mean, double* nu_max, double* nu
     return LBM_OK;
 }
 
-// A kernel may write doubles to p itself: device memory, on 8 bytes.  Anything else goes through a copy,
-// which takes any address and reports a bad one.
-static bool kernel_writes_doubles(const void* p)
-{
-    cudaPointerAttributes a{};
-    if (((uintptr_t)p & 7) != 0) return false;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice;
-}
-
 int lbm_nusselt_profile(lbm_handle h, int face, double* nu, long n, int device_ptrs)
 {
     if (!h || !nu) return fail(h, LBM_EINVAL, "handle or output is NULL");
-    // the face is checked before its length is, and the length before the kernel writes n values
-    const bool fits = face >= 0 && face < 2 * h->dim && n == face_nodes(h, face);
-    const bool direct = device_ptrs && fits && kernel_writes_doubles(nu);
-    int rc = nusselt_common(h, face, direct ? nu : h->nu_profile, h->nu_result);
+    const int rc = nusselt_common(h, face, h->nu_result);
     if (rc) return rc;
-    if (!fits) return fail(h, LBM_EINVAL, "face %d has %ld nodes, not %ld", face, face_nodes(h, face), n);
-    if (!direct)
-        LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double),
-                                  device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+    if (n != face_nodes(h, face)) return fail(h, LBM_EINVAL, "face %d has %ld nodes, not %ld", face, face_nodes(h, face), n);
+    LBM_CK(h, cudaMemcpyAsync(nu, h->nu_profile, n * sizeof(double),
+                              device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
     LBM_CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }

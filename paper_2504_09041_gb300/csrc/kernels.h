@@ -109,7 +109,8 @@ cudaError_t launch_set_pops(int dim, int prec, void* f, void* g, const Geometry&
 // scratch must hold nusselt_scratch_doubles(n_face) doubles plus one unsigned ticket (ticket
 // must be zero on entry and is left zero on exit).  result receives
 // {sum, max, argmax, min, argmin} as doubles.
-// profile may be any device memory, result too, or host memory where host_writes() holds.
+// profile is device memory of the library (a caller's buffer gets a copy, which knows other GPUs and ends
+// of allocations); result likewise, or host memory where host_writes() holds.
 size_t nusselt_scratch_doubles(long n_face);
 // Kernels of the current device may write ordinary host memory (the CPU's page tables serve the GPU, as
 // on Grace-Blackwell): a few result numbers then need no copy of their own.
