@@ -149,7 +149,9 @@ inline cudaError_t launch_step_kernel(void (*kernel)(P...), dim3 grid, dim3 bloc
     cfg.stream = st;
     cfg.attrs = &overlap;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not again by the next launch
+    return e;
 }
 
 template <class R, int QF, int QG>

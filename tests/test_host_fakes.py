@@ -18,6 +18,7 @@ extern "C" {
 void** __cudaRegisterFatBinary(void*) { return nullptr; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction() {}
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaMalloc(void** p, size_t n) { *p = malloc(n); return cudaSuccess; }
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
@@ -107,3 +108,39 @@ def test_wall_profile_reaches_the_caller_by_a_copy(tmp_path):
     serves the one and reports the other, a kernel's store does neither.  So the kernel writes memory of
     the handle and the copy goes to the caller, wherever the pointer is said to be."""
     assert run(tmp_path, "profile", PROFILE, ["api.cu"]) == ["0", "1", "0", "1"]
+
+
+LAUNCH = r"""
+static cudaError_t last = cudaSuccess;
+extern "C" {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**)
+{
+    return last = cudaErrorInvalidConfiguration;
+}
+cudaError_t cudaGetLastError()
+{
+    const cudaError_t e = last;
+    last = cudaSuccess;
+    return e;
+}
+int launch_nothing();
+}
+int main()
+{
+    const int e = launch_nothing();
+    printf("%d %d", e == cudaErrorInvalidConfiguration, cudaGetLastError() == cudaSuccess);
+    return 0;
+}
+"""
+
+
+def test_failed_launch_leaves_no_error_behind(tmp_path):
+    """The launch of a dependent step reports its own error once: the next good call, which ends in
+    cudaGetLastError, must not report it again as its own."""
+    kernel = tmp_path / "nothing.cu"
+    kernel.write_text("""
+#include "kernels.h"
+__global__ void nothing(int) {}
+extern "C" int launch_nothing() { return lbm::launch_step_kernel(nothing, dim3(1), dim3(1), nullptr, 3); }
+""")
+    assert run(tmp_path, "launch", LAUNCH, [str(kernel)]) == ["1", "1"]
