@@ -454,10 +454,11 @@ __device__ __forceinline__ void store_node_f16s(__half* __restrict__ fout, __hal
     }
 }
 
-// 1 / x to about an ulp: the hardware's approximation y and one step of a power series in its residual
-// e = 1 - x y: 1 / x = y (1 + e + e^2 + ...), to order e^2 for double (y has about 20 bits) and to order
-// e for float.  Three FP64 operations instead of the eight or so of an IEEE division, whose last
-// half ulp the velocity does not need.
+// 1 / x within an ulp, for x away from the ends of the range (0 and infinity give NaN): the hardware's
+// approximation y and a Householder step in its residual e = 1 - x y, which is exact to rounding:
+// 1 / x = y (1 + e + e^2 + ...), cubic for double (y has about 20 bits), to order e (Newton's) for
+// float.  Three FP64 operations instead of the eight or so of an IEEE division, whose last half ulp the
+// velocity does not need.
 __device__ __forceinline__ double recip(double x)
 {
     double y;
