@@ -215,18 +215,29 @@ __device__ __forceinline__ void pulled_by_warp(const typename S::T* f, const typ
 // and FP16 storage within two ulps of FP64, on values that carry FP32 rounding).  Where that is no
 // ordinary number (a diverged node's density 0, infinite or NaN) the velocity is the division's.  160^3: FP32 133 us against 644 (floor 125), T alone 69
 // against 228; FP64 1067 against 1622.
-template <class S, int DIM, class Idx, bool kFlow>
+template <class S, int DIM, class Idx, bool kFlow, bool kFlat>
 __global__ void __launch_bounds__(256)
     fields_kernel(const typename S::T* f, const typename S::T* g, Geometry geo, double gbeta, double T_ref,
                   int gaxis, double* rho, double* ux, double* uy, double* uz, double* Tout)
 {
     using R = typename S::R;
     using L = Lat<DIM>;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= geo.nx || y >= geo.ny) return;
-    const int i = x + geo.nx * y + geo.nxy * z;
+    int x, y, z, i;
+    if constexpr (kFlat) {
+        const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+        if (t >= (unsigned)geo.n) return;
+        i = (int)t;
+        z = DIM == 2 ? 0 : i / geo.nxy;
+        const int r = i - z * geo.nxy;
+        y = r / geo.nx;
+        x = r - y * geo.nx;
+    } else {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+        z = blockIdx.z;
+        if (x >= geo.nx || y >= geo.ny) return;
+        i = x + geo.nx * y + geo.nxy * z;
+    }
     R fo[L::QF], go[L::QG];
     pulled_by_warp<S, DIM, Idx>(f, g, geo, R(T_ref), x, y, z, i, fo, go);
     R dT = go[0];
@@ -500,17 +511,38 @@ cudaError_t launch_set_pops(int dim, int prec, void* f, void* g, const Geometry&
     return cudaGetLastError();
 }
 
+template <class S, int D, class Idx>
+static auto fields_instance(bool flow, bool flat)
+{
+    if (flat) return flow ? fields_kernel<S, D, Idx, true, true> : fields_kernel<S, D, Idx, false, true>;
+    return flow ? fields_kernel<S, D, Idx, true, false> : fields_kernel<S, D, Idx, false, false>;
+}
+
+// Threads of the read-out along the linear index instead of along rows, where rows leave lanes idle: an idle
+// lane costs as much as a busy one on the FP64 pipe and on the way to memory.  A warp that spans rows
+// takes the general pull, which FP64, bound by its pipe, does not feel; 3D FP32 and FP16 do, the more
+// of a row's warps would have been interior ones, and 2D a little.  All fields, a million nodes in 3D,
+// 300,000 in 2D, rows -> flat: FP64 nx = 4 2315 -> 306 us, 33 543 -> 294, 100 348 -> 269, 150 276 -> 254, 250
+// even; 3D FP32 4 298 -> 58, 33 84 -> 57, 40 77 -> 60, but 48 51 -> 56, 65 51 -> 54, 160 39 -> 53; 2D FP32 33
+// 21 -> 12.6, 129 14.6 -> 12.5, 300 even (T alone 4.4 -> 5.2).
+static bool fields_flat(const Geometry& g, int prec, int dim)
+{
+    const int lanes = (g.nx + 31) / 32 * 32, idle = lanes - g.nx;
+    return (prec == kF64 ? 32 : (dim == 2 ? 8 : 3)) * idle > lanes;
+}
+
 cudaError_t launch_fields(int dim, int prec, const void* f, const void* g, const Geometry& geo,
                           const HostCoeffs& hc, double* rho, double* ux, double* uy, double* uz,
                           double* T, cudaStream_t st)
 {
-    const dim3 b = block_shape(geo, prec, dim), grid = grid_shape(geo, b);
+    const bool flat = fields_flat(geo, prec, dim);
+    const dim3 b = flat ? dim3(256, 1, 1) : block_shape(geo, prec, dim);
+    const dim3 grid = flat ? dim3((unsigned)(((long long)geo.n + 255) / 256), 1, 1) : grid_shape(geo, b);
     const bool flow = rho || ux || uy || uz;
     LBM_DISPATCH(dim, prec, {
         using TT = typename S::T;
-        auto kern = index32(geo, Lat<D>::QF)
-                        ? (flow ? fields_kernel<S, D, unsigned, true> : fields_kernel<S, D, unsigned, false>)
-                        : (flow ? fields_kernel<S, D, size_t, true> : fields_kernel<S, D, size_t, false>);
+        auto kern = index32(geo, Lat<D>::QF) ? fields_instance<S, D, unsigned>(flow, flat)
+                                             : fields_instance<S, D, size_t>(flow, flat);
         kern<<<grid, b, 0, st>>>((const TT*)f, (const TT*)g, geo, hc.gbeta, hc.T_ref, hc.gaxis, rho, ux, uy, uz, T);
     });
     return cudaGetLastError();
