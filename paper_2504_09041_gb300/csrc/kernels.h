@@ -287,6 +287,18 @@ inline bool flip_pays(const Geometry& g, int q, int prec)
     return 2.0 * q * (double)g.n * (double)storage_bytes(prec) > 129e6;
 }
 
+// FP16 storage, two nodes per thread: rows must fill the pairs' warps about as well as they fill single
+// nodes'.  A pair's warp does the work of num / den one-node warps:
+// - 2D, both buffers in L2, 15 / 8: 1.2 million nodes, pairs against one node, nx = 64 17.5 us against 18.2, 128
+//   16.3 against 17.7; but 32 33.0 against 18.2, 96 21.1 against 18.5, 160 20.5 against 18.1, 258 20.3 against 19.4.
+// - 2D beyond, 8 / 5: 8 million, 64 114 against 124, 130 151 against 155, 322 119 against 139; but 96 133 against 129.
+// - 3D, 7 / 4: 6.4 million, 98 336 against 343, 258 315 against 320; but 32 507 against 289, 96 339 against 287, 160 323
+//   against 288, 194 339 against 328.
+inline bool pairs_fill_rows(int nx, int num, int den)
+{
+    return nx % 2 == 0 && num * ((nx / 2 + 31) / 32) < den * ((nx + 31) / 32);
+}
+
 inline dim3 grid_shape(const Geometry& g, dim3 b)
 {
     return dim3((g.nx + b.x - 1) / b.x, (g.ny + b.y - 1) / b.y, g.nz);

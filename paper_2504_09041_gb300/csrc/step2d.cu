@@ -38,10 +38,13 @@ static cudaError_t run(const void* fin, const void* gin, void* fout, void* gout,
                                       make_unit_coeffs<double, 2>(hc), status);
     }
     if constexpr (std::is_same<S, StoreF16S>::value) {
-        // two nodes per thread where rows start on 4 bytes, in boxes that fill the SMs with them
+        // two nodes per thread where rows start on 4 bytes and fill its warps, in boxes that fill the SMs with them
         const bool aligned = (((uintptr_t)fin | (uintptr_t)gin | (uintptr_t)fout | (uintptr_t)gout) & 3) == 0;
-        if (unit_rates_2d(hc) && block.x == 0 && geo.n >= kPairNodes && geo.nx % 2 == 0 && aligned && step_index32(geo, 9, hc)) {
-            const dim3 b(geo.nx > 64 ? 64 : 32, geo.nx > 64 ? 2 : 4, 1);
+        const bool filled = flip_pays(geo, 18, kF16S) ? pairs_fill_rows(geo.nx, 8, 5) : pairs_fill_rows(geo.nx, 15, 8);
+        if (unit_rates_2d(hc) && block.x == 0 && geo.n >= kPairNodes && filled && aligned && step_index32(geo, 9, hc)) {
+            // (blocks one warp wide where a row's warps are odd in number: nx = 192, 1.2 million nodes 17.5 -> 17.0 us)
+            const bool odd = (geo.nx / 2 + 31) / 32 % 2 != 0;
+            const dim3 b(odd ? 32 : 64, odd ? 4 : 2, 1);
             return launch_step_kernel(step_d2q9_pair_f16s_kernel<unsigned>, dim3((geo.nx / 2 + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1),
                                       b, st, (const __half*)fin, (const __half*)gin, (__half*)fout, (__half*)gout, geo,
                                       make_unit_coeffs<float, 2>(hc), status, flip);

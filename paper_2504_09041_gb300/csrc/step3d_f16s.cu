@@ -17,10 +17,10 @@ static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fou
     using T = typename S::T;
     using R = typename S::R;
     if constexpr (kU == 3) {
-        // two nodes per thread in large boxes (see the kernel) whose rows start on 4 bytes, unless the
-        // caller chose a launch shape of the one-node kernel
+        // two nodes per thread in large boxes (see the kernel) whose rows start on 4 bytes and fill its warps,
+        // unless the caller chose a launch shape of the one-node kernel
         const bool aligned = (((uintptr_t)fin | (uintptr_t)gin | (uintptr_t)fout | (uintptr_t)gout) & 3) == 0;
-        if (geo.n >= 6000000 && geo.nx % 2 == 0 && geo.ny <= 65535 && aligned && block.x == 0 && hc.rows3d == 0 && step_index32(geo, 27, hc)) {
+        if (geo.n >= 6000000 && pairs_fill_rows(geo.nx, 7, 4) && geo.ny <= 65535 && aligned && block.x == 0 && hc.rows3d == 0 && step_index32(geo, 27, hc)) {
             const int warps = (geo.nx / 2 + 31) / 32;
             const dim3 pb(warps & 1 ? 32 : 64, 1, 1);
             step_d3q27_pair_f16s_kernel<unsigned><<<dim3((geo.nx / 2 + pb.x - 1) / pb.x, geo.ny, geo.nz), pb, 0, st>>>(
