@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
                              const typename S::T* __restrict__ g_prev,
                              const RT* __restrict__ mu_in, RT* __restrict__ mu_out, Geometry geo,
                              Coeffs2D<typename S::R> cr, Coeffs2D<TapeT<typename S::R, RT>> c,
-                             int design_face, double* __restrict__ grad)
+                             int design_face, double* __restrict__ grad, bool early)
 {
     using R = typename S::R;
     using RF = TapeT<R, RT>;
@@ -664,6 +664,7 @@ __global__ void __launch_bounds__(kSync ? 256 : 128, kSync ? 2 : 1)
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     const bool active = x < geo.nx && y < geo.ny;
     wait_previous_step();
+    if (early) release_next_step();
     if (!kSync && !active) return;
     x = min(x, geo.nx - 1);
     y = min(y, geo.ny - 1);

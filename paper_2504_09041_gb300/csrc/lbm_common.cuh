@@ -17,15 +17,19 @@ namespace lbm {
 enum FaceKind { kPeriodic = 0, kAdiabatic = 1, kFixedT = 2 };
 
 // 2D steps of one time loop are launched as programmatic dependents (launch_step_kernel): a step's
-// blocks may start while the previous step drains, wait here for it to complete before their first
-// access to populations, and only then let the step after them start, so at most two steps are ever
-// in flight.  That hides the launch (a step of 64^2 nodes: FP64 8.58 -> 8.07 us, FP32 1.86 -> 1.80; 256^2
-// FP32 2.64 -> 2.56).  The 3D steps are launched one after the other: their times do not change, and
-// in FP64 blocks that wait beside running ones share the sub-partitions' FP64 units unevenly (32^3: 67
-// us against 41).
-__device__ __forceinline__ void wait_previous_step()
+// blocks may start once those of the step before it have exited, and wait here for it to complete
+// before their first access to populations, so at most two steps are ever in flight.  That hides the
+// launch (in graphs, 64^2: FP64 5.7 -> 5.4 us, FP32 1.92 -> 1.73; 512^2 FP32 6.0 -> 5.8; in a stream, 64^2 FP32 4.1 ->
+// 2.65).  The 3D steps are launched one after the other: their times do not change.
+__device__ __forceinline__ void wait_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// After the wait: the next step's blocks may start already, beside this one's.  Where a step's blocks take
+// more than half of the GPU's places but not all, those of the next one that find none left crowd onto
+// the SMs that come free first, and the step lasts as long as a full SM's (2D FP32 372 x 277 4.35 us
+// against 3.15 without, 65 x 1000 4.1 against 3.1; FP64 288 x 288 51 against 32); elsewhere the single boxes gain nothing
+// from it, and it is left to adjoint steps that fill the GPU and batches that do not fill it in part.
+__device__ __forceinline__ void release_next_step()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
