@@ -205,7 +205,9 @@ inline auto make_step_coeffs(const HostCoeffs& h)
 //   against 15.8 in blocks of 256 threads on 16; 1024 x 512 takes 189.7 us against 196 (a finer tail).
 //   Above 65535 rows two warps, the launch grid's limit.
 // 2D, FP32 and FP16 storage: 64 x 2 (1024 x 512 FP32 9.97 us against 10.13 for 256 threads, 512^2 5.77
-//   against 5.95, 64^2 1.80 against 2.15; one warp per block runs at 16.9, bound by block turnover).
+//   against 5.95, 64^2 1.80 against 2.15; one warp per block runs at 16.9, bound by block turnover); 96 x 2 for
+//   rows of three warps, of which 64 x 2 leaves a quarter idle (96 x 900 FP32 2.82 us against 3.21, 78 x 1406 3.66
+//   against 4.53, 95 x 13000 29.9 against 31.2).
 // 3D: 64 x 1, which at 72-96 registers per thread lets 10-14 blocks share an SM against four of 256
 //   threads (256^3 FP32: 16.4 against 15.8 GLUPS); 32 x 1 where a row ends in a half-empty block
 //   (131 x 93 x 77: FP32 64.0 us against 68.7, FP16S 45.3 against 51.7, FP64 1273 against 1288);
@@ -218,7 +220,7 @@ inline dim3 block_shape(const Geometry& g, int prec, int dim, dim3 chosen = dim3
     const int rows = g.ny > 65535 ? 2 : 1;
     if (dim == 3) return dim3(warps & 1 ? 32 : (warps & 3 || g.n < (1 << 21) ? 64 : 128), rows, 1);
     if (prec == kF64) return dim3(32, rows, 1);
-    return g.nx > 32 ? dim3(64, 2, 1) : dim3(32, 4, 1);
+    return warps == 1 ? dim3(32, 4, 1) : dim3(warps == 3 ? 96 : 64, 2, 1);
 }
 
 // 32-bit element offsets suffice when every population plane index q * n fits in 32 bits.
