@@ -83,7 +83,7 @@ typedef struct {
     long long steps;            /* time steps taken since creation */
     double bytes_per_node_update; /* algorithmic HBM bytes per node and step: 2 (q_f + q_g) size */
     size_t state_bytes;         /* size of an lbm_get_state checkpoint */
-    int block_x, block_y;       /* thread-block shape of the step launch */
+    int block_x, block_y;       /* thread-block shape of the step launch (tma_rows aside) */
     int graph_steps;            /* steps per CUDA graph replayed by lbm_step (0: plain launches) */
     int g_attractors;           /* energy attractors of orders 3-4: 0 = option A, 1 = option B */
     int fp16_stochastic;        /* LBM_FP16S: 1 = stochastic rounding of the stored deviations */

@@ -547,7 +547,8 @@ int lbm_info(lbm_handle h, lbm_info_t* o)
     o->steps = h->steps;
     o->bytes_per_node_update = 2.0 * (h->qf + h->qg) * (double)lbm::storage_bytes(h->prec);
     o->state_bytes = kStateHeader + pop_bytes(h);
-    const dim3 b = lbm::block_shape(h->geo, h->prec, h->dim, dim3(h->block_x, h->block_y, 1));
+    const dim3 b = lbm::step_shape(h->geo, h->prec, h->dim, h->hc, dim3(h->block_x, h->block_y, 1),
+                                   lbm::starts_on_words(h->f[0], h->g[0], h->f[1], h->g[1])).block;
     o->block_x = (int)b.x;
     o->block_y = (int)b.y;
     o->graph_steps = h->graph_steps;

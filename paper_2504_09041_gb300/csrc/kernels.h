@@ -306,4 +306,42 @@ inline dim3 grid_shape(const Geometry& g, dim3 b)
     return dim3((g.nx + b.x - 1) / b.x, (g.ny + b.y - 1) / b.y, g.nz);
 }
 
+// Which step kernel a box takes, and its thread blocks; on_words: its buffers start on 4 bytes.
+enum StepKind {
+    kStepNode,    // one thread per node
+    kStepSplit,   // 2D FP64: the two lattices of a node on two warps (step_d2q9_split_f64_kernel)
+    kStepPair     // FP16 storage: two nodes per thread (step_d2q9_pair_f16s_kernel, step_d3q27_pair_f16s_kernel)
+};
+struct StepShape {
+    StepKind kind;
+    dim3 block;
+};
+
+constexpr int kPairNodes2D = 300000, kPairNodes3D = 6000000;   // nodes from which boxes fill the SMs with pairs
+constexpr int kSplitWarps = 448;   // warps of 32 nodes up to which two warps per 32 nodes find a sub-partition each
+                                   // (112^2: 7.4 us against 7.6; 128^2: 8.7 against 8.3)
+
+inline StepShape step_shape(const Geometry& g, int prec, int dim, const HostCoeffs& hc, dim3 chosen, bool on_words)
+{
+    const bool reduced = dim == 2 ? unit_rates_2d(hc) : rate_class(hc) == 3;
+    if (reduced && chosen.x == 0 && step_index32(g, dim == 2 ? 9 : 27, hc)) {
+        if (dim == 2 && prec == kF64 && (long long)((g.nx + 31) / 32) * g.ny <= kSplitWarps)
+            return {kStepSplit, dim3(64, 1, 1)};
+        // pairs, one warp wide where a row's warps are odd in number (2D nx = 192, 1.2 million nodes 17.5 -> 17.0 us)
+        const int odd = (g.nx / 2 + 31) / 32 % 2;
+        if (dim == 2 && prec == kF16S && on_words && g.n >= kPairNodes2D &&
+            (flip_pays(g, 18, prec) ? pairs_fill_rows(g.nx, 8, 5) : pairs_fill_rows(g.nx, 15, 8)))
+            return {kStepPair, odd ? dim3(32, 4, 1) : dim3(64, 2, 1)};
+        if (dim == 3 && prec == kF16S && on_words && g.n >= kPairNodes3D && hc.rows3d == 0 && g.ny <= 65535 &&
+            pairs_fill_rows(g.nx, 7, 4))
+            return {kStepPair, dim3(odd ? 32 : 64, 1, 1)};
+    }
+    return {kStepNode, block_shape(g, prec, dim, chosen)};
+}
+
+inline bool starts_on_words(const void* a, const void* b, const void* c, const void* d)
+{
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 3) == 0;
+}
+
 }  // namespace lbm

@@ -16,19 +16,15 @@ static cudaError_t launch_plain_f16s(const void* fin, const void* gin, void* fou
     using S = StoreF16S;
     using T = typename S::T;
     using R = typename S::R;
+    const StepShape shape = step_shape(geo, kF16S, 3, hc, block, starts_on_words(fin, gin, fout, gout));
+    const dim3 b = shape.block;
     if constexpr (kU == 3) {
-        // two nodes per thread in large boxes (see the kernel) whose rows start on 4 bytes and fill its warps,
-        // unless the caller chose a launch shape of the one-node kernel
-        const bool aligned = (((uintptr_t)fin | (uintptr_t)gin | (uintptr_t)fout | (uintptr_t)gout) & 3) == 0;
-        if (geo.n >= 6000000 && pairs_fill_rows(geo.nx, 7, 4) && geo.ny <= 65535 && aligned && block.x == 0 && hc.rows3d == 0 && step_index32(geo, 27, hc)) {
-            const int warps = (geo.nx / 2 + 31) / 32;
-            const dim3 pb(warps & 1 ? 32 : 64, 1, 1);
-            step_d3q27_pair_f16s_kernel<unsigned><<<dim3((geo.nx / 2 + pb.x - 1) / pb.x, geo.ny, geo.nz), pb, 0, st>>>(
+        if (shape.kind == kStepPair) {
+            step_d3q27_pair_f16s_kernel<unsigned><<<dim3((geo.nx / 2 + b.x - 1) / b.x, geo.ny, geo.nz), b, 0, st>>>(
                 (const T*)fin, (const T*)gin, (T*)fout, (T*)gout, geo, make_unit_coeffs<R, 3>(hc), status, flip);
             return cudaGetLastError();
         }
     }
-    const dim3 b = block_shape(geo, kF16S, 3, block);
     const auto c = make_step_coeffs<R, kU>(hc);
     const bool idx32 = step_index32(geo, 27, hc);
     const int rows = idx32 ? rows3d_for(hc) : 1;
