@@ -140,8 +140,8 @@ LBM_API int lbm_set_omegas(lbm_handle h, const double* om_f, int n_f, const doub
  * numbers with a 48-bit significand evaluated on the FP32 pipes; 1 FP64; 0 FP32), "adjoint_fp64" (0 or 1: the same as "adjoint_arith" 0 or 1),
  * "adjoint_sync" (thread blocks of the adjoint kernel: 0 = 64 x 2; 1-4 = 64 x 4, 128 x 2 (the
  * default; 32 x 2 beyond one wave of them), 32 x 4, 64 x 2 whose warps pass a barrier between the phases of the node's work so
- * that they share the instruction fetches of the long unrolled product; results agree to
- * rounding), "adjoint_overlap" (1, the default: lbm_adjoint_step recomputes the next segment's
+ * that they share the instruction fetches of the long unrolled product; 1-4 take
+ * reduced products at the default rates, 0 the general ones; results agree to rounding), "adjoint_overlap" (1, the default: lbm_adjoint_step recomputes the next segment's
  * states on a second, low-priority stream while the adjoint steps of the current one run, with
  * a second set of segment buffers; 0: one stream, one set),
  * "graph_steps" (even count of steps that lbm_step replays as one CUDA graph; 0 disables),
@@ -212,8 +212,9 @@ LBM_API int lbm_set_wall_profile(lbm_handle h, int face, const double* T_w, long
  * K = ceil(sqrt(n_steps)) steps, then n_steps fused adjoint steps backward, recomputing each
  * segment of K states once from its checkpoint: about 2 sqrt(n_steps) states of device memory and
  * one extra forward pass.  The vector-Jacobian products of the collision are evaluated at the
- * recomputed forward intermediates of each node (in the forward step's own register type, FP32
- * for FP32 / FP16 states), with the adjoint carried in double-float arithmetic by default: the
+ * recomputed forward intermediates of each node's general collision (in FP32 for FP32 / FP16
+ * states; FP64 and FP16 states at the default rates are advanced by a reduced collision, the same
+ * function with other rounding), with the adjoint carried in double-float arithmetic by default: the
  * gradient equals the FP64 adjoint's to about 1e-11 relative, at a third of its cost on GPUs whose
  * FP64 rate is a small fraction of their FP32 rate.  lbm_set_param "adjoint_arith" = 1 selects FP64, 0 FP32 (about twice as fast
  * again, gradients to about 1e-4 relative after 2000 steps).  The design gradient is always

@@ -37,9 +37,10 @@ static cudaError_t run_adjoint(const void* f_prev, const void* g_prev, const voi
         const dim3 grid((geo.nx + b.x - 1) / b.x, (geo.ny + b.y - 1) / b.y, 1);
         auto kern = unit_rates_2d(hc) ? adjoint_step_d2q9_kernel<S, RT, true, true> : adjoint_step_d2q9_kernel<S, RT, true>;
         // The next adjoint step's blocks start early (release_next_step) where this one's fill the GPU (512 threads
-        // to an SM): 256^2 FP32 19.8 us against 20.3, 300 x 280 25.9 against 26.9.  With places left they would take
-        // those of the forward steps beside them (200 x 150 18.3 against 16.6), and in FP64, whose steps share
-        // one pipe, they always do (256^2 125 against 120, 200 x 150 98 against 73).
+        // to an SM): FP32 256^2 19.8 us per step of 128, forward passes included, against 20.3, 300 x 280 25.9
+        // against 26.9.  With places left they would take those of the forward steps beside them (200 x 150
+        // 18.3 against 16.6), and in FP64, whose steps share one pipe, they always do (256^2 125 against 120,
+        // 200 x 150 98 against 73).
         const long blocks = (long)grid.x * grid.y, places = 512 / (b.x * b.y);
         const bool early = !std::is_same<S, StoreF64>::value && 20 * ((blocks + 151) / 152) > 17 * places;
         return launch_step_kernel(kern, grid, b, st, (const T*)f_prev, (const T*)g_prev, (const RT*)mu_in, (RT*)mu_out,

@@ -24,11 +24,12 @@
 namespace lbm {
 
 // Reverse-mode products multiply an adjoint value (type RT) by a forward value of the node's
-// collision (type RF).  The forward values are the forward step's own intermediates: for FP32 /
-// FP16 states they are FP32 numbers (RF = float), computed with the same FP32 arithmetic as the
-// forward step, and the products, which carry the adjoint, are formed in RT; for FP64 states
-// RF = RT.  Quantities that depend on forward values only (the Jacobian's entries) are evaluated
-// in RF.
+// collision (type RF).  The forward values are the intermediates of the general collision at the
+// node's state: for FP32 / FP16 states they are FP32 numbers (RF = float), and the products, which
+// carry the adjoint, are formed in RT; for FP64 states RF = RT.  (The forward step computes the same
+// function with them, except that FP64 and FP16 states at the rates lbm_create sets are advanced by
+// the reduced collision, whose rounding differs.)  Quantities that depend on forward values only (the
+// Jacobian's entries) are evaluated in RF.
 template <class R, class RT>
 using TapeT = typename std::conditional<std::is_same<R, float>::value, float, RT>::type;
 

@@ -200,19 +200,20 @@ inline auto make_step_coeffs(const HostCoeffs& h)
 
 // Default thread blocks, x-major so that a warp reads and writes 32 consecutive nodes; a
 // caller-chosen shape (block.x > 0) replaces it.
-// 2D, FP64: one warp, so that few warps spread over all SMs: an SM takes one FP64 warp instruction per 19
-//   cycles and a sub-partition one per 64, so 64^2 nodes (128 warps) take 8.1 us a step on 128 SMs
-//   against 15.8 in blocks of 256 threads on 16; 1024 x 512 takes 189.7 us against 196 (a finer tail).
+// 2D, FP64: one warp, so that few warps spread over all SMs: an SM takes one FP64 warp instruction per 16
+//   cycles and a sub-partition one per 64, so 128^2 nodes (512 warps) take 8.4 us a step against 14.9 in
+//   blocks of 256 threads on 64 SMs; 1024 x 512 takes 176.2 us against 181.8 (a finer tail).
 //   Above 65535 rows two warps, the launch grid's limit.
-// 2D, FP32 and FP16 storage: 64 x 2 (1024 x 512 FP32 9.97 us against 10.13 for 256 threads, 512^2 5.77
-//   against 5.95, 64^2 1.80 against 2.15; one warp per block runs at 16.9, bound by block turnover); 96 x 2 for
+// 2D, FP32 and FP16 storage: 64 x 2 (1024 x 512 FP32 9.91 us against 10.12 for 256 threads, 512^2 5.71
+//   against 5.79, 64^2 1.71 against 1.98; one warp per block 10.5, bound by block turnover); 96 x 2 for
 //   rows of three warps, of which 64 x 2 leaves a quarter idle (96 x 900 FP32 2.82 us against 3.21, 78 x 1406 3.66
 //   against 4.53, 95 x 13000 29.9 against 31.2).
 // 3D: 64 x 1, which at 72-96 registers per thread lets 10-14 blocks share an SM against four of 256
-//   threads (256^3 FP32: 16.4 against 15.8 GLUPS); 32 x 1 where a row ends in a half-empty block
-//   (131 x 93 x 77: FP32 64.0 us against 68.7, FP16S 45.3 against 51.7, FP64 1273 against 1288);
-//   128 x 1 from two million nodes on, where rows fill such blocks (256^3: FP32 849 us against 853,
-//   FP16S 826 against 832; but 64^3 15.8 against 14.5).  Above 65535 rows two rows of them, as in 2D.
+//   threads (256^3 FP32 837 us against 851); 32 x 1 where a row ends in a half-empty block
+//   (131 x 93 x 77: FP32 65.3 us against 68.4, FP16S 45.8 against 53.5, FP64 1292 against 1306);
+//   128 x 1 from two million nodes on, where rows fill such blocks (256^3: FP32 834 us against 837, FP16S one
+//   node per thread 801 against 806; but 64^3 FP32 18.7 against 17.8, FP16S 16.3 against 14.6).  Above 65535 rows
+//   two rows of them, as in 2D.
 inline dim3 block_shape(const Geometry& g, int prec, int dim, dim3 chosen = dim3(0, 0, 0))
 {
     if (chosen.x > 0) return dim3(chosen.x, chosen.y, 1);
@@ -276,8 +277,8 @@ inline int rate_class(const HostCoeffs& h)
 }
 
 // Rows per thread of the 3D FP32 / FP16S step: the handle's setting, or when that is 0 one, the
-// fastest with every collision (FP32 128^3 106 us against 111 for two rows, 256^3 853 against 862,
-// 32^3 4.1 against 5.7; only the general collision at 256^3 is within 0.2 % either way).
+// fastest with every collision (128^3 FP32 107 us against 113 for two rows, FP16S 82 against 85; 256^3 FP32 835
+// against 850; only the general collision at 256^3 is within 0.2 % either way).
 inline int rows3d_for(const HostCoeffs& h) { return h.rows3d > 0 ? h.rows3d : 1; }
 
 // Both buffers of a box exceed the 129 MB L2.  A step that walks the box in the other direction than the one

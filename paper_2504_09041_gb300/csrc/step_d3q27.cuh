@@ -1047,10 +1047,11 @@ __device__ __forceinline__ void pair_node(const float f[27], const float g[15], 
 // without an x component load, and all links store, 32 bits at once; links along x are two 16-bit
 // loads, the second a hit in L1.  The second node waits as packed halves (hold) while the first
 // is computed, so registers stay near one node's (96, no spills; 80 and 112 measured slower).
-// 256^3: 798 -> 677 us per step (26 % -> 31 % of HBM bandwidth reading and writing each value once);
-// where L2 serves part of the loads the one-node kernel is faster (128^3 79 against 96 us, 160^3 166
-// against 207), so boxes take this one from 6 million nodes on (192^3: 302 against 325).
-// Needs an even nx (then rows and planes start on 4 bytes).  The results are bitwise those of the
+// 256^3: 801 -> 680 us per step (52 % -> 61 % of the measured copy bandwidth); issue slots are then 59 %
+// busy, and the first stalls are memory latency and the fetch of the two nodes' unrolled code (1.8 and 1.7
+// warps per issue, ncu at 192^3).  Where L2 serves part of the loads the one-node kernel is faster (128^3 79
+// against 96 us, 160^3 169 against 207), so boxes take this one from 6 million nodes on (192^3: 305
+// against 328), if rows fill its warps (pairs_fill_rows).  Rows and planes start on 4 bytes.  The results are bitwise those of the
 // one-node kernel.
 template <class Idx>
 __global__ void __maxnreg__(LBM_MAXREG3D_PAIR)
